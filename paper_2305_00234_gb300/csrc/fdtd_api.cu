@@ -239,6 +239,9 @@ void validate(const fdtd_grid_desc& d)
             if (!std::isfinite(d.src_wave[s])) arg_error("non-finite source waveform sample");
 }
 
+// Elements of a DFT snapshot slot: three components of nd samples, padded to 16 bytes (bulk copies).
+size_t snap_stride(size_t nd, size_t ts) { return (3 * nd * ts + 15) / 16 * 16 / ts; }
+
 size_t footprint(const fdtd_grid_desc& d, const int ptot[3])
 {
     const size_t ts = d.precision == 64 ? 8 : 4;
@@ -261,7 +264,7 @@ size_t footprint(const fdtd_grid_desc& d, const int ptot[3])
     b += (d.density_layout == 1 ? 3 : 1) * nd * ts;                  // rho (per component with layout 1)
     for (int k = 0; k < 3; ++k) b += nd * (size_t)ptot[k] * 2 * ts;   // Q
     b += 2 * nd * 3 * (size_t)d.n_freq * 16;                          // forward + adjoint DFT
-    b += (size_t)fdtd::kMaxSnap * 3 * nd * ts + nv * 8;               // DFT snapshot ring, staging
+    b += (size_t)fdtd::kMaxSnap * snap_stride(nd, ts) * ts + nv * 8;               // DFT snapshot ring, staging
     b += nv * 8 + ((nv + 255) / 256 + 1) * 8;                         // gradient + partials
     b += ((size_t)d.n_steps + 1) * d.n_freq * 2 * ts;                 // phase table
     b += (size_t)d.n_steps * (2 * fdtd::kMaxBasis + 2) * ts;          // source waves, TF/SF tables
@@ -475,8 +478,8 @@ struct Solver : SolverBase {
                 encode_map(&maps[par].e, par ? fld[2] : fld[0], kSYE);
                 encode_map(&maps[par].h, par ? fld[3] : fld[1], kSYH);
             }
-            CK(fdtd::prepare_step<T>());
         }
+        CK(fdtd::prepare_step<T>());
         // CPML tables {1/kappa, b, c, 0} per slab index
         for (int a = 0; a < 3; ++a) {
             const int W = p.W[a];
@@ -538,7 +541,8 @@ struct Solver : SolverBase {
             CK(cudaMemcpyAsync(phase, ph.data(), ph.size() * sizeof(V2), cudaMemcpyHostToDevice, c->work));
         }
         p.K = fdtd::kMaxSnap;
-        snap = talloc((size_t)fdtd::kMaxSnap * 3 * c->nd);
+        p.snap_stride = (long long)snap_stride(c->nd, sizeof(T));
+        snap = talloc((size_t)fdtd::kMaxSnap * p.snap_stride);
         p.snap = snap;
         staging = c->alloc(std::max<size_t>(std::max(c->nd, c->nvar), 1) * sizeof(double));
         for (int m = 0; m < 2; ++m) {
@@ -546,6 +550,7 @@ struct Solver : SolverBase {
             dp[m].nf = d.n_freq;
             dp[m].K = fdtd::kMaxSnap;
             dp[m].snap = snap;
+            dp[m].snap_stride = p.snap_stride;
             dp[m].dft = dft[m];
             dp[m].ph = phase;
         }
@@ -1019,11 +1024,13 @@ struct Solver : SolverBase {
         pm_fwd.gap_hist = pm_gh;
         pm_fwd.nsamp = (int)(3 * c->ngap);
         pm_fwd.snap = pm_he;
+        pm_fwd.snap_stride = 3 * (long long)c->nd;
         pm_fwd.K = C;
         pm_fwd.snap0 = 0;
         // recompute pass: design-box E^{n+1} into slots 1.., the pole term into pm_hq
         pm_rec = pf;
         pm_rec.snap = pm_he + 3 * c->nd;
+        pm_rec.snap_stride = 3 * (long long)c->nd;
         pm_rec.hist_dq = pm_hq;
         pm_rec.K = C;
         // adjoint pass: second state set, direct drive table at the gap samples
@@ -1048,6 +1055,7 @@ struct Solver : SolverBase {
         std::memcpy(pm_adj.sb, base.gb, sizeof pm_adj.sb);
         pm_adj.tfsf_i0 = -1;
         pm_adj.snap = pm_ha + 3 * c->nd;
+        pm_adj.snap_stride = 3 * (long long)c->nd;
         pm_adj.K = C;
     }
 
@@ -1067,7 +1075,7 @@ struct Solver : SolverBase {
         CK(cudaStreamSynchronize(c->work));
         if (h[2] & 4) {
             c->dead = true;
-            throw Err{FDTD_ERR_TIMEOUT, "a wait of the step kernel gave up after its time limit"};
+            throw Err{FDTD_ERR_TIMEOUT, "a wait of the step or DFT kernel gave up after its time limit"};
         }
         if (h[2] & 1) {
             c->dead = true;
@@ -1421,7 +1429,7 @@ struct Solver : SolverBase {
         CK(cudaStreamSynchronize(c->work));
         if (hctl[2] & 4) {
             c->dead = true;
-            throw Err{FDTD_ERR_TIMEOUT, "a wait of the step kernel gave up after its time limit"};
+            throw Err{FDTD_ERR_TIMEOUT, "a wait of the step or DFT kernel gave up after its time limit"};
         }
         if (hctl[2] & 1) {
             c->dead = true;

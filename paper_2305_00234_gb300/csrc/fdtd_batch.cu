@@ -79,7 +79,7 @@ __device__ __forceinline__ void dft_voxel_lean(const DParams<T>& d, long long v,
         for (int f = 0; f < d.nf; ++f) {
             T re = T(0), im = T(0);
             for (int s = 0; s < cnt; ++s) {
-                const T e = __ldcg(sp + (long long)((n0 + s) % d.K) * 3 * d.nd);
+                const T e = __ldcg(sp + (long long)((n0 + s) % d.K) * d.snap_stride);
                 const auto ph = __ldg(d.ph + (long long)(n0 + s + 1) * d.nf + f);
                 re = fma(e, ph.x, re);
                 im = fma(-e, ph.y, im);

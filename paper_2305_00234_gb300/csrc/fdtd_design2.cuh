@@ -40,7 +40,7 @@ __device__ __forceinline__ float design_pair_column(const KParams<float>& p, con
     const bool col_scalar = p.td_acc || p.hist_dq || i < p.mb[C][0] || i + 1 >= p.mb[C][1] || j < p.mb[C][2] ||
                             j >= p.mb[C][3] || (C == 2 && (i == p.tfsf_i0 || i + 1 == p.tfsf_i0)) ||
                             ((C == 1 || C == 2) && i == 0) || (C != 1 && j == 0);
-    const long long slot0 = (long long)((n - p.snap0) % p.K) * 3 * p.nd + C * p.nd;
+    const long long slot0 = (long long)((n - p.snap0) % p.K) * p.snap_stride + C * p.nd;
     const int P = p.P[C], P1 = p.P1[C];
     const float2 idx2 = f2(p.inv_dx, p.inv_dx), one2 = f2(1.f, 1.f);
     const float2 D1 = f2(p.D1[C], p.D1[C]), dD = f2(p.dD[C], p.dD[C]), N1 = f2(p.N1[C], p.N1[C]),

@@ -2,6 +2,7 @@
 #include <utility>
 
 #include "fdtd_design2.cuh"
+#include "fdtd_dft.cuh"
 #include "fdtd_kernels.cuh"
 #include "fdtd_launch.h"
 #include "fdtd_shell2.cuh"
@@ -114,6 +115,8 @@ int pole_bucket(int max_poles)
 template <typename T>
 cudaError_t prepare_step()
 {
+    const cudaError_t e = cudaFuncSetAttribute(dft_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DftSmem<T>::total);
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(step_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)StepSmem<T>::total);
 }
 
@@ -185,10 +188,15 @@ cudaError_t graph_e_design(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T
 }
 
 template <typename T>
+static dim3 dft_grid(const DParams<T>& d)
+{
+    return dim3((unsigned)((3 * d.nd + kDftChunk - 1) / kDftChunk));
+}
+
+template <typename T>
 cudaError_t graph_dft(cudaGraph_t g, cudaGraphNode_t* node, const DParams<T>& d, int cnt)
 {
-    return graph_kernel(g, node, dft_kernel<T>, dim3((unsigned)((d.nd + kReduceThreads - 1) / kReduceThreads)),
-                        dim3(kReduceThreads), 0, d, cnt);
+    return graph_kernel(g, node, dft_kernel<T>, dft_grid(d), dim3(kDftThreads), DftSmem<T>::total, d, cnt);
 }
 
 template <typename T>
@@ -271,8 +279,7 @@ template <typename T>
 cudaError_t launch_dft(const DParams<T>& d, int cnt, cudaStream_t s, bool pdl)
 {
     if (d.nd == 0 || cnt <= 0) return cudaSuccess;
-    return launch_chain(dft_kernel<T>, dim3((unsigned)((d.nd + kReduceThreads - 1) / kReduceThreads)),
-                        dim3(kReduceThreads), 0, s, pdl, d, cnt);
+    return launch_chain(dft_kernel<T>, dft_grid(d), dim3(kDftThreads), DftSmem<T>::total, s, pdl, d, cnt);
 }
 
 

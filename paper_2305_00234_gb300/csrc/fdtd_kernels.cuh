@@ -7,7 +7,7 @@
 //                    both materials weighted by 1-rho and rho (Eqs. (Maxwells)a,b, (eps_mixed),
 //                    (sigma_mixed), (Poles_mixed)), the pole recursion
 //                    Q <- Q + (alpha-1) Q + beta (E^{n+1}+E^n), and an E snapshot for the DFT;
-// and, every kMaxSnap steps, dft_kernel: the running FP64 DFT over the design box.  The gradient
+// and, every kMaxSnap steps, dft_kernel (fdtd_dft.cuh): the running FP64 DFT over the design box.  The gradient
 // kernel evaluates the structure of Eq. (Gradient_analytic) per voxel (or per E sample with the
 // per-sample density layout) with a deterministic warp-shuffle reduction of its squared norm.
 //
@@ -238,9 +238,6 @@ constexpr int ed_min_blocks()
 
 // L2 prefetch (no registers held) of a line a coming plane's update reads.
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-#ifndef FDTD_DFT_PF
-#define FDTD_DFT_PF 1   // 1: dft_voxel prefetches its accumulators into L2 first (config 2: 0.243 -> 0.212 ms)
-#endif
 #ifndef FDTD_ED_PF
 #define FDTD_ED_PF 0   // planes ahead in e_design_column (0: none)
 #endif
@@ -263,7 +260,7 @@ __device__ __forceinline__ T e_design_column(const KParams<T>& p, const PoleTabl
     const long long dcol = (long long)(j - p.db[2]) * p.dnx + (i - p.db[0]);
     const bool inxy_m = i >= p.mb[C][0] && i < p.mb[C][1] && j >= p.mb[C][2] && j < p.mb[C][3];
     const bool inxy_g = i >= p.gb[0] && i < p.gb[1] && j >= p.gb[2] && j < p.gb[3];
-    const long long slot0 = (long long)((n - p.snap0) % p.K) * 3 * p.nd + C * p.nd;
+    const long long slot0 = (long long)((n - p.snap0) % p.K) * p.snap_stride + C * p.nd;
     const T hinc_n = (C == 2 && i == p.tfsf_i0) ? __ldg(p.hinc + n) * p.inv_dx : T(0);
     T emax = T(0);
     for (int kb = k0; kb < k1; kb += PZ) {
@@ -353,64 +350,6 @@ __global__ void __launch_bounds__(kBX * kBY, ed_min_blocks<T, MP>()) e_design_ke
         if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
     }
     finish_step(p.ctl, p.nblocks_e, n);
-}
-
-// ---------------------------------------------------------------------------------------------
-// Blocked running DFT over the design box.  After cnt steps n0..n0+cnt-1 (n0 = ctl[0] - cnt), each
-// thread owns one design voxel: it reads the cnt snapshots E^{n+1} of its three samples, forms the
-// block sums sum_s E^{n0+s+1} (cos, -sin)(w_f (n0+s+1) dt) in the accumulation type A, and adds
-// them to the FP64 accumulators, which are read and written once per block instead of every step.
-// ---------------------------------------------------------------------------------------------
-// The fold of one voxel v: steps n0 .. n0 + cnt - 1 (cnt <= kMaxSnap).
-template <typename T, bool CG>
-__device__ __forceinline__ void dft_voxel(const DParams<T>& d, long long v, int n0, int cnt)
-{
-#if FDTD_DFT_PF
-    if constexpr (!CG)   // the FP64 accumulators into L2 while the snapshots load
-        for (int q = 0; q < 3 * d.nf; ++q) prefetch_l2(d.dft + (long long)q * d.nd + v);
-#endif
-    T e[kMaxSnap][3];
-#pragma unroll
-    for (int s = 0; s < kMaxSnap; ++s) {
-        if (s < cnt) {
-            const T* sp = d.snap + (long long)((n0 + s) % d.K) * 3 * d.nd + v;
-            e[s][0] = ldf<CG>(sp);
-            e[s][1] = ldf<CG>(sp + d.nd);
-            e[s][2] = ldf<CG>(sp + 2 * d.nd);
-        }
-    }
-    for (int f = 0; f < d.nf; ++f) {
-        T re[3] = {T(0), T(0), T(0)}, im[3] = {T(0), T(0), T(0)};
-#pragma unroll
-        for (int s = 0; s < kMaxSnap; ++s) {
-            if (s < cnt) {
-                const auto ph = __ldg(d.ph + (long long)(n0 + s + 1) * d.nf + f);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    re[c] = fma(e[s][c], ph.x, re[c]);
-                    im[c] = fma(-e[s][c], ph.y, im[c]);
-                }
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            double2* acc = d.dft + (long long)(f * 3 + c) * d.nd + v;
-            double2 a = ldf<CG>(acc);
-            a.x += (double)re[c];
-            a.y += (double)im[c];
-            *acc = a;
-        }
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kReduceThreads) dft_kernel(const DParams<T> d, int cnt)
-{
-    pdl_wait();                                   // the snapshots of the block's last step
-    pdl_trigger();
-    const long long v = (long long)blockIdx.x * kReduceThreads + threadIdx.x;
-    if (v >= d.nd) return;
-    dft_voxel<T, false>(d, v, __ldcg(d.ctl) - cnt, cnt);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -151,7 +151,8 @@ struct KParams {
     cpx<T>* Q[3];                // pole currents [P[c]][nd]
     int K;                       // snapshot ring length (steps per DFT block)
     int snap0;                   // step n writes its E^{n+1} snapshot to slot (n - snap0) mod K
-    T* snap;                     // E snapshots of the design box [K][3][nd]
+    T* snap;                     // E snapshots of the design box [K][3][nd], slots snap_stride apart
+    long long snap_stride;
     int nb;                      // point-source basis functions (0 = none)
     int src_direct;              // 1: the drive of source-box sample s at step n is src_wave[n * nsamp + s]
     int nsamp;                   //    (s = local voxel * 3 + component), no basis expansion
@@ -194,10 +195,11 @@ template <typename T>
 struct DParams {
     long long nd;
     int nf, K;
-    const T* snap;                          // [K][3][nd]
+    const T* snap;                          // [K][3][nd], slots snap_stride (a multiple of 16 bytes) apart
+    long long snap_stride;
     double2* dft;                           // [nf][3][nd]
     const typename vec2_of<T>::type* ph;    // (cos, sin)(w_f n dt) in T, [(M+1)][nf]
-    const int* ctl;
+    int* ctl;                               // of the step kernels
 };
 
 template <typename T>
