@@ -559,13 +559,10 @@ struct Solver : SolverBase {
         p.ctl = ctl;
         for (int m = 0; m < 2; ++m) dp[m].ctl = ctl;
         shell.pair = shell_pairable(p) ? 1 : 0;
-        p.nblocks_s = fdtd::shell_blocks(shell);
+        fdtd::shell_blocks(shell);
         p.edz = 1;
         p.ed_pair = design_pairable() ? 1 : 0;
-        p.nblocks_d = c->nd ? fdtd::design_blocks(p.ed_pair ? c->dn[0] / 2 : c->dn[0], c->dn[1], c->dn[2], p.edz,
-                                                  FDTD_ED_FLAT && !p.ed_pair)
-                            : 0;
-        p.nblocks_e = p.nblocks_s + p.nblocks_d;
+        if (c->nd) p.edz = fdtd::design_planes((p.ed_pair ? c->dn[0] / 2 : c->dn[0]) * c->dn[1], c->dn[2]);
         p.blowup = (T)1e30;
         p.n_steps = d.n_steps;
         p.tfsf_i0 = -1;
@@ -870,7 +867,7 @@ struct Solver : SolverBase {
 
     // One whole time step: the H phase (shell H next to the interior kernel when concurrent), then
     // the E phase, whose shell E and design E kernels write disjoint cells and run side by side when
-    // concurrent (the last block of the two advances the step counter).
+    // concurrent.
     cudaError_t launch_one_step(const KParams<T>& q, int parity, bool concurrent, const StepMaps* mp = nullptr)
     {
         if (!concurrent || c->nd == 0) {
@@ -893,11 +890,13 @@ struct Solver : SolverBase {
         return e;
     }
 
-    // Parameters of a step with the given parity: odd steps read the second buffer of each pair.
-    KParams<T> par(const KParams<T>& p, int parity) const
+    // Parameters of a step with the given parity (odd steps read the second buffer of each pair), off
+    // steps after the device step counter.
+    KParams<T> par(const KParams<T>& p, int parity, int off = 0) const
     {
-        if (!(parity & 1)) return p;
         KParams<T> q = p;
+        q.n_off = off;
+        if (!(parity & 1)) return q;
         for (int cc = 0; cc < 3; ++cc) {
             std::swap(q.E[cc], q.En[cc]);
             std::swap(q.H[cc], q.Hn[cc]);
@@ -1062,9 +1061,10 @@ struct Solver : SolverBase {
     void pm_steps(const KParams<T>& p, const StepMaps* mp, int n_from, int n_to)
     {
         for (int s = n_from; s < n_to; ++s) {
-            const KParams<T> q = par(p, s);
+            const KParams<T> q = par(p, s, s - n_from);
             CK(launch_one_step(q, s, true, mp));   // both phases on two streams, as in the captured graphs
         }
+        if (n_to > n_from) CK(fdtd::launch_block_end(p.ctl, n_to - n_from, c->work));
         c->tim.launches += (long long)(n_to - n_from) * (fused ? 4 : 3);
     }
 
@@ -1286,7 +1286,7 @@ struct Solver : SolverBase {
             prev = cur;
         };
         for (int st = 0; st < steps && e == cudaSuccess; ++st) {
-            const KParams<T> q = par(p, st);
+            const KParams<T> q = par(p, st, st);
             phase([&] {
                 cudaGraphNode_t n = nullptr;
                 if (e == cudaSuccess && has_shell && (e = fdtd::graph_shell<T>(g, &n, q, shell, false)) == cudaSuccess)
@@ -1301,11 +1301,17 @@ struct Solver : SolverBase {
                     cur.push_back(n);
             });
         }
-        if (e == cudaSuccess && c->nd)
+        cudaGraphNode_t begin = nullptr, dftn = nullptr;
+        if (e == cudaSuccess) e = fdtd::graph_block_begin(g, &begin, p.ctl);
+        if (e == cudaSuccess)
             phase([&] {
                 cudaGraphNode_t n = nullptr;
-                if ((e = fdtd::graph_dft<T>(g, &n, dp[mode], steps)) == cudaSuccess) cur.push_back(n);
+                if (c->nd && (e = fdtd::graph_dft<T>(g, &dftn, dp[mode], steps)) == cudaSuccess) cur.push_back(dftn);
+                if (e == cudaSuccess && (e = fdtd::graph_block_end(g, &n, p.ctl, steps)) == cudaSuccess) cur.push_back(n);
             });
+        // the copy for the DFT comes before both the DFT and the step advance
+        for (cudaGraphNode_t to : cur)
+            if (e == cudaSuccess) e = cudaGraphAddDependencies(g, &begin, &to, nullptr, 1);
         cudaGraphExec_t ex = nullptr;
         if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
         cudaGraphDestroy(g);
@@ -1329,12 +1335,12 @@ struct Solver : SolverBase {
         const KParams<T>& p = mode ? pa : pf;
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(c->work, cudaStreamCaptureModeThreadLocal));
-        cudaError_t err = cudaSuccess;
+        cudaError_t err = fdtd::launch_block_begin(p.ctl, c->work);
         for (int s = 0; s < steps && err == cudaSuccess; ++s) {   // graphs start at even steps
-            const KParams<T> q = par(p, s);
+            const KParams<T> q = par(p, s, s);
             err = launch_one_step(q, s, true);
         }
-        if (err == cudaSuccess) err = fdtd::launch_dft<T>(dp[mode], steps, c->work);
+        if (err == cudaSuccess) err = end_block(mode, steps);
         cudaError_t e2 = cudaStreamEndCapture(c->work, &g);
         if (err != cudaSuccess || e2 != cudaSuccess) {
             if (g) cudaGraphDestroy(g);
@@ -1345,6 +1351,13 @@ struct Solver : SolverBase {
         cudaGraphDestroy(g);
         CK(err);
         graph[mode][which] = ex;
+    }
+
+    // The launches that end a block of steps: the DFT fold, the step advance.
+    cudaError_t end_block(int mode, int steps)
+    {
+        const cudaError_t e = fdtd::launch_dft<T>(dp[mode], steps, c->work);
+        return e == cudaSuccess ? fdtd::launch_block_end(base.ctl, steps, c->work) : e;
     }
 
     void run(int mode)
@@ -1374,8 +1387,9 @@ struct Solver : SolverBase {
             const int cnt = b < full ? K : rem;
             if (c->prof && b % kProfEvery == 0) {
                 sampled.push_back(b);
+                CK(fdtd::launch_block_begin(ctl, c->work));
                 for (int q = 0; q < cnt; ++q, ++s) {
-                    const KParams<T> pp = par(p, s);
+                    const KParams<T> pp = par(p, s, q);
                     cudaEvent_t* e = &c->ev[5 * (size_t)s];
                     CK(cudaEventRecord(e[0], c->work));
                     CK(fdtd::launch_shell<T>(pp, shell, false, c->work));
@@ -1387,7 +1401,7 @@ struct Solver : SolverBase {
                     CK(fdtd::launch_e_design<T>(pp, htab, bucket, c->work));
                     CK(cudaEventRecord(e[4], c->work));
                 }
-                CK(fdtd::launch_dft<T>(dp[mode], cnt, c->work));
+                CK(end_block(mode, cnt));
                 CK(cudaEventRecord(c->ev[5 * (size_t)M + b], c->work));
             } else {
                 CK(cudaGraphLaunch(graph[mode][b < full ? 0 : 1], c->work));

@@ -1,4 +1,4 @@
-// Blocked running DFT over the design box.  After cnt steps n0..n0+cnt-1 (n0 = ctl[0] - cnt), the block sums
+// Blocked running DFT over the design box.  After cnt steps n0..n0+cnt-1 (n0 = ctl[3]), the block sums
 // sum_s E^{n0+s+1} (cos, -sin)(w_f (n0+s+1) dt) are formed in T and added to the FP64 accumulators, which
 // are read and written once per block of steps instead of every step.
 //
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kDftThreads, sizeof(T) == 4 ? 5 : 2) dft_kerne
     }
     pdl_wait();                                    // the snapshots of the block's last step
     pdl_trigger();
-    const int n0 = __ldcg(d.ctl) - cnt;
+    const int n0 = __ldcg(d.ctl + 3);
     if (tid == 0) {
         // slots are padded to a multiple of 16 bytes, so the last chunk's copy may be rounded up to one
         const unsigned bytes = ((unsigned)len * (unsigned)sizeof(T) + 15u) / 16u * 16u;

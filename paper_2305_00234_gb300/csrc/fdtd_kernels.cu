@@ -155,16 +155,14 @@ cudaError_t graph_shell(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& 
                   : graph_kernel(g, node, shell_h_kernel<T>, grid, b, 0, p, s);
 }
 
-// Grid of the design-E kernel: one block per (p.edz planes, component) of 32 x 8 columns (32 x 8 column
-// pairs for the paired kernel).
+// Grid of the design-E kernel: one block per (p.edz planes, component) of 256 columns (column pairs for
+// the paired kernel) in row order.
 template <typename T>
 static dim3 design_grid(const KParams<T>& p)
 {
-    const dim3 g3 = grid3((p.db[1] - p.db[0]) / (p.ed_pair ? 2 : 1), p.db[3] - p.db[2], p.db[5] - p.db[4]);
-    const unsigned nxy = (unsigned)(p.db[1] - p.db[0]) * (unsigned)(p.db[3] - p.db[2]);
-    if (FDTD_ED_FLAT && !p.ed_pair)
-        return dim3((nxy + kBX * kBY - 1) / (kBX * kBY), 1, 3 * ((g3.z + p.edz - 1) / p.edz));
-    return dim3(g3.x, g3.y, 3 * ((g3.z + p.edz - 1) / p.edz));
+    const unsigned nxy = (unsigned)((p.db[1] - p.db[0]) / (p.ed_pair ? 2 : 1)) * (unsigned)(p.db[3] - p.db[2]);
+    const unsigned nz = (unsigned)(p.db[5] - p.db[4]);
+    return dim3((nxy + kBX * kBY - 1) / (kBX * kBY), 1, 3 * ((nz + p.edz - 1) / p.edz));
 }
 
 template <typename T>
@@ -199,11 +197,22 @@ cudaError_t graph_dft(cudaGraph_t g, cudaGraphNode_t* node, const DParams<T>& d,
     return graph_kernel(g, node, dft_kernel<T>, dft_grid(d), dim3(kDftThreads), DftSmem<T>::total, d, cnt);
 }
 
-template <typename T>
-unsigned step_blocks(const KParams<T>& p)
+// One thread each: the first step of a block of steps for its DFT launch, and the step counter moved on.
+__global__ void block_begin_kernel(int* ctl) { ctl[3] = ctl[0]; }
+__global__ void block_end_kernel(int* ctl, int cnt)
 {
-    return (unsigned)((p.ib[1] - p.ib[0] + kTX - 1) / kTX) * (unsigned)((p.ib[3] - p.ib[2] + kTY - 1) / kTY) *
-           (unsigned)((p.ib[5] - p.ib[4] + p.kc - 1) / p.kc);
+    pdl_wait();
+    ctl[0] += cnt;
+}
+
+cudaError_t graph_block_begin(cudaGraph_t g, cudaGraphNode_t* node, int* ctl)
+{
+    return graph_kernel(g, node, block_begin_kernel, dim3(1), dim3(1), 0, ctl);
+}
+
+cudaError_t graph_block_end(cudaGraph_t g, cudaGraphNode_t* node, int* ctl, int cnt)
+{
+    return graph_kernel(g, node, block_end_kernel, dim3(1), dim3(1), 0, ctl, cnt);
 }
 
 template <typename T>
@@ -222,11 +231,10 @@ constexpr unsigned kMinColumnBlocks = 2 * 152;
 #ifndef FDTD_SHELL_MINCOLS
 #define FDTD_SHELL_MINCOLS kMinColumnBlocks
 #endif
-unsigned shell_blocks(ShellBoxes& s)
+void shell_blocks(ShellBoxes& s)
 {
-    unsigned t = 0;
     for (s.kz = kShellKZ;; s.kz -= kShellPZ) {
-        t = 0;
+        unsigned t = 0;
         for (int q = 0; q < s.n; ++q) {
             const int* B = s.b[q];
             s.first[q] = t;
@@ -236,7 +244,6 @@ unsigned shell_blocks(ShellBoxes& s)
         s.first[s.n] = t;
         if (t >= FDTD_SHELL_MINCOLS || s.kz <= kShellPZ) break;
     }
-    return t;
 }
 
 template <typename T>
@@ -283,22 +290,30 @@ cudaError_t launch_dft(const DParams<T>& d, int cnt, cudaStream_t s, bool pdl)
 }
 
 
+cudaError_t launch_block_begin(int* ctl, cudaStream_t s)
+{
+    block_begin_kernel<<<1, 1, 0, s>>>(ctl);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_block_end(int* ctl, int cnt, cudaStream_t s)
+{
+    block_end_kernel<<<1, 1, 0, s>>>(ctl, cnt);
+    return cudaGetLastError();
+}
+
 // Columns of kEdZ planes, halved while the launch has fewer than FDTD_ED_MINCOLS blocks (default: one
 // wave of five resident blocks per SM; measured 3.7% faster than two blocks per SM on the 96 x 170 x 170
 // paper grid, whose design box is 26 cells deep in x).
 #ifndef FDTD_ED_MINCOLS
 #define FDTD_ED_MINCOLS (5 * 152)
 #endif
-unsigned design_blocks(int dnx, int dny, int dnz, int& edz, bool flat)
+int design_planes(int columns, int dnz)
 {
-    const dim3 g = grid3(dnx, dny, dnz);
-    const unsigned gxy = flat ? ((unsigned)dnx * (unsigned)dny + kBX * kBY - 1) / (kBX * kBY) : g.x * g.y;
-    unsigned t = 0;
-    for (edz = kEdZ;; edz = (edz + 1) / 2) {
-        t = gxy * 3 * ((g.z + edz - 1) / edz);
-        if (t >= FDTD_ED_MINCOLS || edz == 1) break;
-    }
-    return t;
+    const unsigned gxy = ((unsigned)columns + kBX * kBY - 1) / (kBX * kBY);
+    int edz = kEdZ;
+    while (edz > 1 && gxy * 3 * (((unsigned)dnz + edz - 1) / edz) < FDTD_ED_MINCOLS) edz = (edz + 1) / 2;
+    return edz;
 }
 
 template <typename T>
@@ -388,7 +403,6 @@ cudaError_t launch_rho_scatter(const void* src, int dtype, long long n, const lo
 
 #define FDTD_INSTANTIATE(T)                                                                              \
     template cudaError_t prepare_step<T>();                                                              \
-    template unsigned step_blocks<T>(const KParams<T>&);                                                \
     template cudaError_t graph_step<T>(cudaGraph_t, cudaGraphNode_t*, const KParams<T>&, const StepMaps&); \
     template cudaError_t graph_shell<T>(cudaGraph_t, cudaGraphNode_t*, const KParams<T>&, const ShellBoxes&, bool); \
     template cudaError_t graph_e_design<T>(cudaGraph_t, cudaGraphNode_t*, const KParams<T>&, const PoleTable<T>&, int); \

@@ -14,9 +14,13 @@
 // Thread layout of the per-cell kernels: blocks of (32, 8) threads over (x, y); x is the fastest
 // array axis, so each warp reads and writes 128 contiguous bytes per field (FP32).
 //
-// The step index n lives in device memory (ctl[0]) so that a captured CUDA graph of K steps can be
-// replayed: every kernel reads it, and the last block of the E phase (the shell-E and design-E
-// launches, counted together) advances it.
+// The step index lives in device memory so that a CUDA graph of K steps can be replayed: ctl[0] is the
+// first step of the graph and every launch's step is ctl[0] + n_off (a launch parameter).  Next to the first
+// step, block_begin_kernel copies ctl[0] to ctl[3], where the DFT launch at the end reads it; next to the
+// DFT, block_end_kernel moves ctl[0] on by the graph's steps.  Two one-thread launches a graph, off its
+// critical path, instead of a counter that every block of every E phase adds to behind a fence and a block
+// barrier (1-2 us a step on small grids).  (A conditional store at the end of the shell H kernel instead
+// slowed it from 0.063 to 0.066 ms on a 256^3 grid.)
 #pragma once
 #include "fdtd_params.h"
 
@@ -130,14 +134,14 @@ __device__ __forceinline__ cpx<T> ldg_c(const cpx<T>* p)
 // constant-bank operands).
 // dq (paper mode): sum_p dkappa_p/drho Re{Q_p^{n+1} - Q_p^n} of this sample (-1 for m1's poles,
 // +1 for m2's), the pole term of Eq. (Gradient_FDTD).
-template <typename T, int MP, int C, bool CG = false>
+template <typename T, int MP, int C>
 __device__ __forceinline__ void design_load(const KParams<T>& p, long long dv, cpx<T> (&q)[MP > 0 ? MP : 1])
 {
     const int P = p.P[C];
-    const cpx<T>* __restrict__ Q = p.Q[C];
+    const cpx<T>* Q = p.Q[C];
 #pragma unroll
     for (int pp = 0; pp < MP; ++pp)
-        if (pp < P) q[pp] = ldf<CG>(Q + pp * p.nd + dv);
+        if (pp < P) q[pp] = ld_pre(Q + pp * p.nd + dv);
 }
 
 template <typename T, int MP, int C>
@@ -190,32 +194,39 @@ __device__ __forceinline__ T point_drive(const KParams<T>& p, int i, int j, int 
     return s;
 }
 
+// Step of this launch.  ctl[0] does not change while the step kernels of its graph run, so it may be read
+// before pdl_wait.
 template <typename T>
-__device__ __forceinline__ int read_step(const int* ctl) { return __ldcg(ctl); }
+__device__ __forceinline__ int read_step(const KParams<T>& p) { return __ldcg(p.ctl) + p.n_off; }
 
 // Programmatic dependent launch.  In the step graphs the kernels of a phase depend on those of the phase
 // before through programmatic edges: a kernel's blocks may be launched before its predecessors have
 // finished; pdl_wait() blocks until every predecessor has completed and its memory is visible, and
 // pdl_trigger() lets the successors' blocks be launched once every block of this kernel has issued it.
-// Every kernel of the step graphs waits first and triggers right after, so the next phase's blocks are
-// already resident when a phase drains.  Both are no-ops for an ordinary launch.
+// Every kernel of the step graphs triggers right after its wait, so the next phase's blocks are already
+// resident when a phase drains.  Both are no-ops for an ordinary launch.
+//
+// Loads before the wait.  A phase's blocks start once every block of the phase before has triggered, that
+// is, has passed its own wait: the phase two before is then complete and its stores are performed.  So a
+// kernel may read, ahead of its wait, what only phases two or more before it write, which is most of its
+// own-cell state: the H phase reads H^{n-1/2}, psi_H (the E phase before it writes E, psi_E, Q, the
+// snapshots), the E phase E^n, psi_E, rho, Q (the H phase before it writes H, psi_H).  Those loads bypass
+// L1 (ld_pre) and nothing is stored before the wait.  Their latency then overlaps the drain of the phase
+// before instead of following it.  With the step counter above, a step of a 48^3 grid took 10.3 us before
+// and 7.4 us after, of a 75 x 61 x 83 grid 16.3 and 12.7 us; grids that fill the memory system are unchanged.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// The last block of the launch that owns the step advance moves the device step counter on.
-__device__ __forceinline__ void finish_step(int* ctl, unsigned nblocks, int n)
+template <typename T>
+__device__ __forceinline__ T ld_pre(const T* p) { return __ldcg(p); }
+template <typename T>
+__device__ __forceinline__ cpx<T> ld_pre(const cpx<T>* p)
 {
-    __syncthreads();
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
-        __threadfence();
-        const unsigned prev = atomicAdd((unsigned*)(ctl + 1), 1u);
-        if (prev == nblocks - 1) {
-            ctl[1] = 0;
-            atomicExch(ctl, n + 1);
-            __threadfence();
-        }
-    }
+    using V = typename vec2_of<T>::type;
+    const V v = __ldcg(reinterpret_cast<const V*>(p));
+    return cpx<T>{v.x, v.y};
 }
+
 
 // ---------------------------------------------------------------------------------------------
 // E update inside the working box.  A thread owns one component c of the (x, y) column of a block
@@ -225,7 +236,7 @@ __device__ __forceinline__ void finish_step(int* ctl, unsigned nblocks, int n)
 // included) before any store: blended CCPR update of the design samples, background
 // update of the gap samples and of samples outside their component's sample box, point sources,
 // the E snapshot for the blocked DFT and the paper-mode records.  The working box lies outside the
-// CPML, so there is no psi here.  Owns the step advance.
+// CPML, so there is no psi here.
 template <typename T, int MP>
 constexpr int ed_min_blocks()
 {
@@ -236,14 +247,9 @@ constexpr int ed_min_blocks()
 #endif
 }
 
-// L2 prefetch (no registers held) of a line a coming plane's update reads.
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-#ifndef FDTD_ED_PF
-#define FDTD_ED_PF 0   // planes ahead in e_design_column (0: none)
-#endif
-
 // One component C of the (x, y) column (i, j), planes [k0, k1); returns max |E| of its samples.
-template <typename T, int MP, int C, bool CG = false>
+// PDL: the caller has not waited for the phase before; the first batch's own-sample loads come first.
+template <typename T, int MP, int C, bool CG = false, bool PDL = false>
 __device__ __forceinline__ T e_design_column(const KParams<T>& p, const PoleTable<T>& tab, int i, int j, int k0, int k1, int n)
 {
     constexpr int PZ = kEdPZ;
@@ -252,10 +258,10 @@ __device__ __forceinline__ T e_design_column(const KParams<T>& p, const PoleTabl
     constexpr int ca = C == 0 ? 2 : C - 1, cb = C == 2 ? 0 : C + 1;
     const unsigned oa = C == 0 ? (unsigned)p.nx : (C == 1 ? (unsigned)p.plane : 1u);
     const unsigned ob = C == 0 ? (unsigned)p.plane : (C == 1 ? 1u : (unsigned)p.nx);
-    const T* __restrict__ Ha = p.Hn[ca];   // H^{n+1/2}, just written by the H update
-    const T* __restrict__ Hb = p.Hn[cb];
-    const T* __restrict__ Ec = p.E[C];     // E^n
-    const T* __restrict__ rc = p.rhoc[C];
+    const T* Ha = p.Hn[ca];   // H^{n+1/2}, just written by the H update
+    const T* Hb = p.Hn[cb];
+    const T* Ec = p.E[C];     // E^n
+    const T* rc = p.rhoc[C];
     const unsigned plane = (unsigned)p.plane, col = (unsigned)j * (unsigned)p.nx + (unsigned)i;
     const long long dcol = (long long)(j - p.db[2]) * p.dnx + (i - p.db[0]);
     const bool inxy_m = i >= p.mb[C][0] && i < p.mb[C][1] && j >= p.mb[C][2] && j < p.mb[C][3];
@@ -274,28 +280,25 @@ __device__ __forceinline__ T e_design_column(const KParams<T>& p, const PoleTabl
             if (k >= k1) continue;
             const unsigned id = (unsigned)k * plane + col;
             const long long dv = (long long)(k - p.db[4]) * p.dplane + dcol;
+            e0[r] = ld_pre(Ec + id);
+            ds[r] = inxy_m && k >= p.mb[C][4] && k < p.mb[C][5] && !(inxy_g && k >= p.gb[4] && k < p.gb[5]);
+            rho[r] = ds[r] ? ld_pre(rc + dv) : T(0);
+            if (ds[r]) design_load<T, MP, C>(p, dv, q[r]);
+        }
+        if (PDL && kb == k0) {
+            pdl_wait();
+            pdl_trigger();
+        }
+#pragma unroll
+        for (int r = 0; r < PZ; ++r) {
+            const int k = kb + r;
+            if (k >= k1) continue;
+            const unsigned id = (unsigned)k * plane + col;
             const int la = C == 0 ? j : (C == 1 ? k : i), lb = C == 0 ? k : (C == 1 ? i : j);
             ha[r] = ldf<CG>(Ha + id);
             hb[r] = ldf<CG>(Hb + id);
             ham[r] = la > 0 ? ldf<CG>(Ha + id - oa) : T(0);
             hbm[r] = lb > 0 ? ldf<CG>(Hb + id - ob) : T(0);
-            if constexpr (!CG && FDTD_ED_PF > 0) {   // the rows of a coming plane into L2
-                if (k + FDTD_ED_PF < k1) {
-                    const unsigned ip = id + FDTD_ED_PF * plane;
-                    const long long dp = dv + FDTD_ED_PF * p.dplane;
-                    prefetch_l2(Ha + ip);
-                    prefetch_l2(Hb + ip);
-                    prefetch_l2(Ec + ip);
-                    prefetch_l2(rc + dp);
-#pragma unroll
-                    for (int pp = 0; pp < (MP > 0 ? MP : 1); ++pp)
-                        if (pp < p.P[C]) prefetch_l2(p.Q[C] + pp * p.nd + dp);
-                }
-            }
-            e0[r] = ldf<CG>(Ec + id);
-            ds[r] = inxy_m && k >= p.mb[C][4] && k < p.mb[C][5] && !(inxy_g && k >= p.gb[4] && k < p.gb[5]);
-            rho[r] = ds[r] ? ldf<CG>(rc + dv) : T(0);
-            if (ds[r]) design_load<T, MP, C, CG>(p, dv, q[r]);
         }
 #pragma unroll
         for (int r = 0; r < PZ; ++r) {
@@ -328,28 +331,17 @@ template <typename T, int MP>
 __global__ void __launch_bounds__(kBX * kBY, ed_min_blocks<T, MP>()) e_design_kernel(const KParams<T> p, const PoleTable<T> tab)
 {
     const int zc = blockIdx.z / 3, c = blockIdx.z - 3 * zc;
-    int i, j;
-    if (FDTD_ED_FLAT) {   // columns in row order, kBX * kBY per block
-        const int dnx = p.db[1] - p.db[0];
-        const int col = blockIdx.x * (kBX * kBY) + threadIdx.y * kBX + threadIdx.x;
-        const int y = col / dnx;
-        i = p.db[0] + (col - y * dnx);
-        j = p.db[2] + y;
-    } else {
-        i = p.db[0] + blockIdx.x * kBX + threadIdx.x;
-        j = p.db[2] + blockIdx.y * kBY + threadIdx.y;
-    }
+    const int dnx = p.db[1] - p.db[0];   // columns in row order, kBX * kBY per block
+    const int col = blockIdx.x * (kBX * kBY) + threadIdx.y * kBX + threadIdx.x;
+    const int y = col / dnx;
+    const int i = p.db[0] + (col - y * dnx), j = p.db[2] + y;
     const int k0 = p.db[4] + zc * p.edz, k1 = min(p.db[5], k0 + p.edz);
-    pdl_wait();
-    pdl_trigger();
-    const int n = read_step<T>(p.ctl);
-    if (i < p.db[1] && j < p.db[3]) {
-        const T emax = c == 0 ? e_design_column<T, MP, 0>(p, tab, i, j, k0, k1, n)
-                     : c == 1 ? e_design_column<T, MP, 1>(p, tab, i, j, k0, k1, n)
-                              : e_design_column<T, MP, 2>(p, tab, i, j, k0, k1, n);
-        if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
-    }
-    finish_step(p.ctl, p.nblocks_e, n);
+    const int n = read_step(p);
+    if (j >= p.db[3]) return;
+    const T emax = c == 0 ? e_design_column<T, MP, 0, false, true>(p, tab, i, j, k0, k1, n)
+                 : c == 1 ? e_design_column<T, MP, 1, false, true>(p, tab, i, j, k0, k1, n)
+                          : e_design_column<T, MP, 2, false, true>(p, tab, i, j, k0, k1, n);
+    if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
 }
 
 // ---------------------------------------------------------------------------------------------

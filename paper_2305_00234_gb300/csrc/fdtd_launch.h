@@ -11,8 +11,6 @@ int pole_bucket(int max_poles);
 template <typename T>
 cudaError_t prepare_step();
 // pdl: launch as a programmatic dependent launch in the step chain (see pdl_wait in fdtd_kernels.cuh)
-template <typename T>
-unsigned step_blocks(const KParams<T>& p);
 // kernel nodes of a step graph, without dependencies
 template <typename T>
 cudaError_t graph_step(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& p, const StepMaps& m);
@@ -22,16 +20,21 @@ template <typename T>
 cudaError_t graph_e_design(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& p, const PoleTable<T>& tab, int bucket);
 template <typename T>
 cudaError_t graph_dft(cudaGraph_t g, cudaGraphNode_t* node, const DParams<T>& d, int cnt);
+// begin and end of a block of cnt steps: the first step for the DFT launch, the step counter moved on
+cudaError_t graph_block_begin(cudaGraph_t g, cudaGraphNode_t* node, int* ctl);
+cudaError_t graph_block_end(cudaGraph_t g, cudaGraphNode_t* node, int* ctl, int cnt);
+cudaError_t launch_block_begin(int* ctl, cudaStream_t s);
+cudaError_t launch_block_end(int* ctl, int cnt, cudaStream_t s);
 template <typename T>
 cudaError_t launch_step(const KParams<T>& p, const StepMaps& m, cudaStream_t s, bool pdl = false);
 template <typename T>
 cudaError_t launch_e_design(const KParams<T>& p, const PoleTable<T>& tab, int bucket, cudaStream_t s, bool pdl = false);
 template <typename T>
 cudaError_t launch_dft(const DParams<T>& d, int cnt, cudaStream_t s, bool pdl = false);
-unsigned shell_blocks(ShellBoxes& s);   // fills s.first, returns the launch's blocks
+void shell_blocks(ShellBoxes& s);   // fills s.kz and s.first
 template <typename T>
 cudaError_t launch_shell(const KParams<T>& p, const ShellBoxes& s, bool e_part, cudaStream_t st, bool pdl = false);
-unsigned design_blocks(int dnx, int dny, int dnz, int& edz, bool flat);   // also picks the column depth
+int design_planes(int columns, int dnz);   // z planes per thread of the design-E kernel
 template <typename T>
 cudaError_t launch_grad(const GParams<T>& g, unsigned nblocks, cudaStream_t s);
 cudaError_t launch_gap_gather(const double2* dft, long long nd, int nf, const int* db, int dnx, int dny, const int* gb,

@@ -34,12 +34,6 @@ constexpr int kMaxSnap = 16;      // steps per blocked DFT update (snapshot ring
 #endif
 constexpr int kEdZ = FDTD_ED_Z;     // most z planes per thread in the design-E kernel
 constexpr int kEdPZ = FDTD_ED_PZ;   // of which loaded per batch
-// FDTD_ED_FLAT 1 (default): the one-sample design-E kernel takes (x, y) columns 256 at a time in row order
-// (every lane busy on working boxes narrower than 32 cells: the paper grid's 26-cell-deep box, design E
-// 0.0220 -> 0.0213 ms); 0: 32 x 8 column tiles
-#ifndef FDTD_ED_FLAT
-#define FDTD_ED_FLAT 1
-#endif
 constexpr int kShellPZ = FDTD_SHELL_PZ;   // z planes per batch of loads in the shell kernels
 constexpr int kShellKZ = FDTD_SHELL_KZ;   // most z planes per thread in the shell kernels (a multiple of kShellPZ)
 constexpr int kKC = FDTD_KC;      // z planes per block of the fused step kernel
@@ -166,15 +160,14 @@ struct KParams {
     const T* einc;               // E_inc^n at x = i0 dx
     const T* hinc;               // H_inc^{n+1/2} at x = (i0 - 1/2) dx
     int n_steps;                 // steps of a run
-    int* ctl;                    // [0] step n, [1] finished blocks of the advancing launch, [2] flags
+    int* ctl;                    // [0] first step of the current block of steps, [2] flags, [3] the first step for
+                                 // the block's DFT launch
+    int n_off;                   // the launch's step is ctl[0] + n_off
     int ib[6];                   // interior box of the fused step kernel (empty: x0 = x1)
-    unsigned nblocks_s;          // blocks of the background-E shell kernel
-    unsigned nblocks_d;          // blocks of e_design_kernel
     int edz;                     // z planes per thread of e_design_kernel (<= kEdZ)
     int kc;                      // z planes per block of step_kernel (<= kKC)
     int ed_pair;                 // 1: e_design2_kernel (FP32, x-adjacent sample pairs; nx and the working box's
                                  // x origin and extent even, one density per voxel)
-    unsigned nblocks_e;          // blocks of the E phase (shell E + design E); the last one advances the step
     T blowup;
     long long stall_ns;          // failure-path test hook (step_kernel): > 0 makes block (0, 0, 0) at step 0 wait
                                  // this long on an mbarrier that nothing completes; 0 = off

@@ -39,6 +39,7 @@ __device__ __forceinline__ float2 p_add(float2 a, float2 b) { return __fadd2_rn(
 __device__ __forceinline__ void pf_l2(const float* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 ldp(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ float2 ldp_pre(const float* p) { return __ldcg(reinterpret_cast<const float2*>(p)); }
 __device__ __forceinline__ void stp(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
 
 // The pair (x, x+1), x = B[0] + 2j, of block b / thread t of a paired shell launch (boxes counted in pairs).
@@ -84,12 +85,12 @@ __device__ __forceinline__ void psi_load_p(float* const (&ps)[3][2], const PsiCo
 {
     const unsigned q1 = k * pc.qys + pc.qy0, q2 = (unsigned)max(sz, 0) * plane + col, q0 = k * pc.qxs + pc.qx0;
     const float2 z = f2(0.f, 0.f);
-    v[0] = sy >= 0 ? ldp(ps[0][0] + q1) : z;
-    v[1] = sy >= 0 ? ldp(ps[2][1] + q1) : z;
-    v[2] = sz >= 0 ? ldp(ps[0][1] + q2) : z;
-    v[3] = sz >= 0 ? ldp(ps[1][0] + q2) : z;
-    v[4] = sx >= 0 ? ldp(ps[1][1] + q0) : z;
-    v[5] = sx >= 0 ? ldp(ps[2][0] + q0) : z;
+    v[0] = sy >= 0 ? ldp_pre(ps[0][0] + q1) : z;
+    v[1] = sy >= 0 ? ldp_pre(ps[2][1] + q1) : z;
+    v[2] = sz >= 0 ? ldp_pre(ps[0][1] + q2) : z;
+    v[3] = sz >= 0 ? ldp_pre(ps[1][0] + q2) : z;
+    v[4] = sx >= 0 ? ldp_pre(ps[1][1] + q0) : z;
+    v[5] = sx >= 0 ? ldp_pre(ps[2][0] + q0) : z;
 }
 
 __device__ __forceinline__ void psi_store_p(float* const (&ps)[3][2], const PsiCol& pc, unsigned k, unsigned plane,
@@ -116,12 +117,10 @@ __device__ __forceinline__ void psi_store_p(float* const (&ps)[3][2], const PsiC
 __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_h2_kernel(const KParams<float> p, const ShellBoxes s)
 {
     constexpr int P = kShell2PZ;
-    pdl_wait();
-    pdl_trigger();
     ShellCol cl;
     if (!shell_pair(s, cl)) return;
     const int x = cl.x, y = cl.y;
-    const int n = read_step<float>(p.ctl);
+    const int n = read_step(p);
     const float cneg = -(p.ch * p.inv_dx), idx = p.inv_dx, ch = p.ch;
     const float2 cn = f2(cneg, cneg), idx2 = f2(idx, idx), ch2 = f2(ch, ch);
     const float einc_n = p.tfsf_i0 >= 0 ? __ldg(p.einc + n) : 0.f;
@@ -134,11 +133,11 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_h2_kernel(c
     const bool xp = x + 2 < p.nx, yp = y + 1 < p.ny;
     const unsigned nx = (unsigned)p.nx, plane = (unsigned)p.plane, col = (unsigned)y * nx + (unsigned)x;
     const PsiCol pc = psi_col(p, x, y, sx, sy);
-    const float* __restrict__ E0 = p.E[0];
-    const float* __restrict__ E1 = p.E[1];
-    const float* __restrict__ E2 = p.E[2];
+    const float* E0 = p.E[0];
+    const float* E1 = p.E[1];
+    const float* E2 = p.E[2];
     const float2 z2 = f2(0.f, 0.f);
-    float2 exc = ldp(E0 + (unsigned)cl.k0 * plane + col), eyc = ldp(E1 + (unsigned)cl.k0 * plane + col);
+    float2 exc, eyc;
     for (int it = 0; it < kShellKZ / P; ++it) {
         const int kb = cl.k0 + it * P;
         if (kb >= cl.k1) break;
@@ -148,6 +147,23 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_h2_kernel(c
         for (int r = 0; r < P; ++r) {
             const int k = kb + r;
             sz[r] = slab_index(k, p.cpl[2], p.cph[2], p.nz);
+            if (k >= cl.k1) continue;
+            if (it > 0) continue;
+            const unsigned id = (unsigned)k * plane + col;
+            ho[r][0] = ldp_pre(p.H[0] + id);
+            ho[r][1] = ldp_pre(p.H[1] + id);
+            ho[r][2] = ldp_pre(p.H[2] + id);
+            psi_load_p(p.psiH, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
+        }
+        if (it == 0) {
+            pdl_wait();
+            pdl_trigger();
+            exc = ldp(E0 + (unsigned)kb * plane + col);
+            eyc = ldp(E1 + (unsigned)kb * plane + col);
+        }
+#pragma unroll
+        for (int r = 0; r < P; ++r) {
+            const int k = kb + r;
             if (k >= cl.k1) continue;
             const unsigned id = (unsigned)k * plane + col;
             const bool zp = k + 1 < p.nz;
@@ -172,10 +188,12 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_h2_kernel(c
             exy[r] = yp ? ldp(E0 + id + nx) : z2;
             exz[r] = zp ? ldp(E0 + id + plane) : z2;
             eyz[r] = zp ? ldp(E1 + id + plane) : z2;
-            ho[r][0] = ldp(p.H[0] + id);
-            ho[r][1] = ldp(p.H[1] + id);
-            ho[r][2] = ldp(p.H[2] + id);
-            psi_load_p(p.psiH, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
+            if (it > 0) {
+                ho[r][0] = ldp_pre(p.H[0] + id);
+                ho[r][1] = ldp_pre(p.H[1] + id);
+                ho[r][2] = ldp_pre(p.H[2] + id);
+                psi_load_p(p.psiH, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
+            }
         }
 #pragma unroll
         for (int r = 0; r < P; ++r) {
@@ -221,16 +239,14 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_h2_kernel(c
 }
 
 // E of the shell cells outside the working box, one pair of columns per thread.  It may run concurrently
-// with the design-E kernel: the last block of the two launches advances the step.
+// with the design-E kernel.
 __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_e2_kernel(const KParams<float> p, const ShellBoxes s)
 {
     constexpr int P = kShell2PZ;
-    pdl_wait();
-    pdl_trigger();
     ShellCol cl;
-    const bool live = shell_pair(s, cl);
-    const int n = read_step<float>(p.ctl);
-    if (live) {
+    if (!shell_pair(s, cl)) return;
+    const int n = read_step(p);
+    {
         const int x = cl.x, y = cl.y;
         const float hinc_n = p.tfsf_i0 >= 0 ? __ldg(p.hinc + n) : 0.f;
         const bool check = (n & 15) == 0 || n + 1 == p.n_steps;
@@ -253,14 +269,10 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_e2_kernel(c
             cbi[c] = f2(p.bg_cbi[c], p.bg_cbi[c]);
             cb[c] = f2(p.bg_cb[c], p.bg_cb[c]);
         }
-        const float* __restrict__ H0 = p.Hn[0];
-        const float* __restrict__ H1 = p.Hn[1];
-        const float* __restrict__ H2 = p.Hn[2];
+        const float* H0 = p.Hn[0];
+        const float* H1 = p.Hn[1];
+        const float* H2 = p.Hn[2];
         float2 hxb = z2, hyb = z2;   // H_x, H_y of the plane below the batch
-        if (cl.k0 > 0) {
-            hxb = ldp(H0 + (unsigned)(cl.k0 - 1) * plane + col);
-            hyb = ldp(H1 + (unsigned)(cl.k0 - 1) * plane + col);
-        }
         float emax = 0.f;
         for (int kb = cl.k0; kb < cl.k1; kb += P) {
             float2 h[P][3], hzy[P], hxy[P], hzx[P], hyx[P], e0[P][3], ps[P][6];
@@ -273,6 +285,24 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_e2_kernel(c
                 const bool in_dz = k >= p.db[4] && k < p.db[5];
                 on0[r] = k < cl.k1 && !(in_dx0 && in_dz);
                 on1[r] = k < cl.k1 && !(in_dx1 && in_dz);
+                if (k >= cl.k1) continue;
+                const unsigned id = (unsigned)k * plane + col;
+                e0[r][0] = ldp_pre(p.E[0] + id);
+                e0[r][1] = ldp_pre(p.E[1] + id);
+                e0[r][2] = ldp_pre(p.E[2] + id);
+                psi_load_p(p.psiE, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
+            }
+            if (kb == cl.k0) {
+                pdl_wait();
+                pdl_trigger();
+                if (kb > 0) {
+                    hxb = ldp(H0 + (unsigned)(kb - 1) * plane + col);
+                    hyb = ldp(H1 + (unsigned)(kb - 1) * plane + col);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < P; ++r) {
+                const int k = kb + r;
                 if (k >= cl.k1) continue;
                 const unsigned id = (unsigned)k * plane + col;
                 if (FDTD_SHELL2_PF_E > 0 && k + FDTD_SHELL2_PF_E < cl.k1) {
@@ -291,10 +321,6 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_e2_kernel(c
                 hxy[r] = y > 0 ? ldp(H0 + id - nx) : z2;                  // H_x(y-1)
                 hzx[r] = f2(x > 0 ? H2[id - 1] : 0.f, h[r][2].x);        // H_z(x-1)
                 hyx[r] = f2(x > 0 ? H1[id - 1] : 0.f, h[r][1].x);        // H_y(x-1)
-                e0[r][0] = ldp(p.E[0] + id);
-                e0[r][1] = ldp(p.E[1] + id);
-                e0[r][2] = ldp(p.E[2] + id);
-                psi_load_p(p.psiE, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
             }
 #pragma unroll
             for (int r = 0; r < P; ++r) {
@@ -368,7 +394,6 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_e2_kernel(c
         }
         if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
     }
-    finish_step(p.ctl, p.nblocks_e, n);
 }
 
 }  // namespace fdtd

@@ -358,9 +358,7 @@ __global__ void __launch_bounds__(kPX * kTY, StepCfg<T>::MINB)
     const int k_first = kb - 1;            // >= 0: the interior box starts above plane 0
     const int ne_tot = ke - k_first + 1;   // E planes k_first .. ke
     const int nh_tot = ke - k_first;       // H planes k_first .. ke-1
-    pdl_wait();
-    pdl_trigger();
-    const int n = read_step<T>(p.ctl);
+    const int n = read_step(p);
     auto eslot = [&](int s) { return (T*)((unsigned char*)sE + s * S::e_slot); };
     auto hslot = [&](int s) { return (T*)((unsigned char*)sHo + s * S::h_slot); };
     auto issue_e = [&](int r) {
@@ -380,10 +378,12 @@ __global__ void __launch_bounds__(kPX * kTY, StepCfg<T>::MINB)
     // a block that starts after another one timed out does nothing (the run is already failed)
     const bool skip = __syncthreads_or(tid == 0 && (__ldcg(p.ctl + 2) & 4));
     int e_issued = 0, h_issued = 0;        // meaningful in thread 0
-    if (tid == 0 && !skip) {
-        for (; e_issued < NE && e_issued < ne_tot; ++e_issued) issue_e(e_issued);
+    if (tid == 0 && !skip)                 // H^{n-1/2} was complete before the E phase that is draining now
         for (; h_issued < NH && h_issued < nh_tot; ++h_issued) issue_h(h_issued);
-    }
+    pdl_wait();
+    pdl_trigger();
+    if (tid == 0 && !skip)
+        for (; e_issued < NE && e_issued < ne_tot; ++e_issued) issue_e(e_issued);
     const T cneg = -(p.ch * p.inv_dx);
     const T einc_n = p.tfsf_i0 >= 0 ? __ldg(p.einc + n) : T(0);
     const T hinc_n = p.tfsf_i0 >= 0 ? __ldg(p.hinc + n) : T(0);
@@ -530,17 +530,17 @@ __device__ __forceinline__ PsiCol psi_col(const KParams<T>& p, int x, int y, int
 // psi of one cell for the six curl terms (0 outside the slabs): [0] d/dy of the x row, [1] d/dy of
 // the z row (y slab); [2] d/dz of the x row, [3] d/dz of the y row (z slab); [4] d/dx of the y row,
 // [5] d/dx of the z row (x slab).
-template <typename T, bool CG>
+template <typename T>
 __device__ __forceinline__ void psi_load(T* const (&ps)[3][2], const PsiCol& pc, unsigned k, unsigned plane,
                                          unsigned col, int sx, int sy, int sz, T (&v)[6])
 {
     const unsigned q1 = k * pc.qys + pc.qy0, q2 = (unsigned)max(sz, 0) * plane + col, q0 = k * pc.qxs + pc.qx0;
-    v[0] = sy >= 0 ? ldf<CG>(ps[0][0] + q1) : T(0);
-    v[1] = sy >= 0 ? ldf<CG>(ps[2][1] + q1) : T(0);
-    v[2] = sz >= 0 ? ldf<CG>(ps[0][1] + q2) : T(0);
-    v[3] = sz >= 0 ? ldf<CG>(ps[1][0] + q2) : T(0);
-    v[4] = sx >= 0 ? ldf<CG>(ps[1][1] + q0) : T(0);
-    v[5] = sx >= 0 ? ldf<CG>(ps[2][0] + q0) : T(0);
+    v[0] = sy >= 0 ? ld_pre(ps[0][0] + q1) : T(0);
+    v[1] = sy >= 0 ? ld_pre(ps[2][1] + q1) : T(0);
+    v[2] = sz >= 0 ? ld_pre(ps[0][1] + q2) : T(0);
+    v[3] = sz >= 0 ? ld_pre(ps[1][0] + q2) : T(0);
+    v[4] = sx >= 0 ? ld_pre(ps[1][1] + q0) : T(0);
+    v[5] = sx >= 0 ? ld_pre(ps[2][0] + q0) : T(0);
 }
 
 template <typename T>
@@ -578,8 +578,9 @@ __device__ __forceinline__ T stretch_v(T d, const T* __restrict__ tab, int s, T&
 // the shell, CPML psi_H included.  Within a batch every load is issued before any store (the buffers
 // it writes are not the ones it reads); E_x, E_y of the plane above a batch carry over as the next
 // batch's own.  CG: state loads bypass L1 (for a persistent kernel whose earlier work items on the
-// same SM may hold stale lines).
-template <typename T, bool CG>
+// same SM may hold stale lines).  PDL: the caller has not waited for the phase before; the first batch's
+// H and psi_H loads come first.
+template <typename T, bool CG, bool PDL = false>
 __device__ __forceinline__ void h_column(const KParams<T>& p, int x, int y, int k0, int k1, int n)
 {
     constexpr int P = kShellPZ;
@@ -590,10 +591,10 @@ __device__ __forceinline__ void h_column(const KParams<T>& p, int x, int y, int 
     const bool xp = x + 1 < p.nx, yp = y + 1 < p.ny;
     const unsigned nx = (unsigned)p.nx, plane = (unsigned)p.plane, col = (unsigned)y * nx + (unsigned)x;
     const PsiCol pc = psi_col(p, x, y, sx, sy);
-    const T* __restrict__ E0 = p.E[0];
-    const T* __restrict__ E1 = p.E[1];
-    const T* __restrict__ E2 = p.E[2];
-    T exc = ldf<CG>(E0 + (unsigned)k0 * plane + col), eyc = ldf<CG>(E1 + (unsigned)k0 * plane + col);
+    const T* E0 = p.E[0];
+    const T* E1 = p.E[1];
+    const T* E2 = p.E[2];
+    T exc, eyc;
     for (int it = 0; it < kShellKZ / P; ++it) {   // compile-time trip bound; k1 may end the column early
         const int kb = k0 + it * P;
         if (kb >= k1) break;
@@ -606,6 +607,24 @@ __device__ __forceinline__ void h_column(const KParams<T>& p, int x, int y, int 
             sz[r] = slab_index(k, p.cpl[2], p.cph[2], p.nz);
             if (k >= k1) continue;
             const unsigned id = (unsigned)k * plane + col;
+            a[r].hox = ld_pre(p.H[0] + id);
+            a[r].hoy = ld_pre(p.H[1] + id);
+            a[r].hoz = ld_pre(p.H[2] + id);
+            psi_load(p.psiH, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
+        }
+        if (it == 0) {
+            if (PDL) {
+                pdl_wait();
+                pdl_trigger();
+            }
+            exc = ldf<CG>(E0 + (unsigned)k0 * plane + col);
+            eyc = ldf<CG>(E1 + (unsigned)k0 * plane + col);
+        }
+#pragma unroll
+        for (int r = 0; r < P; ++r) {
+            const int k = kb + r;
+            if (k >= k1) continue;
+            const unsigned id = (unsigned)k * plane + col;
             const bool zp = k + 1 < p.nz;
             a[r].ex0 = r == 0 ? exc : a[r - 1].exz;
             a[r].ey0 = r == 0 ? eyc : a[r - 1].eyz;
@@ -616,10 +635,6 @@ __device__ __forceinline__ void h_column(const KParams<T>& p, int x, int y, int 
             a[r].eyx = xp ? ldf<CG>(E1 + id + 1) : T(0);
             a[r].exz = zp ? ldf<CG>(E0 + id + plane) : T(0);
             a[r].eyz = zp ? ldf<CG>(E1 + id + plane) : T(0);
-            a[r].hox = ldf<CG>(p.H[0] + id);
-            a[r].hoy = ldf<CG>(p.H[1] + id);
-            a[r].hoz = ldf<CG>(p.H[2] + id);
-            psi_load<T, CG>(p.psiH, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
         }
 #pragma unroll
         for (int r = 0; r < P; ++r) {
@@ -665,17 +680,16 @@ __device__ __forceinline__ void h_column(const KParams<T>& p, int x, int y, int 
 template <typename T>
 __global__ void __launch_bounds__(kBX * kBY, sizeof(T) == 8 ? 2 : FDTD_SHELL_MINB) shell_h_kernel(const KParams<T> p, const ShellBoxes s)
 {
-    pdl_wait();
-    pdl_trigger();
     ShellCol cl;
-    if (shell_cell(s, cl)) h_column<T, false>(p, cl.x, cl.y, cl.k0, cl.k1, read_step<T>(p.ctl));
+    if (shell_cell(s, cl)) h_column<T, false, true>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
 }
 
 // E^{n+1} of the cells of one column (x, y), planes [k0, k1), that lie outside the working box, from
 // H^{n+1/2} of the whole grid (after every H update of the step); loads first within a batch, like
 // h_column, with H_x, H_y of the plane below a batch carried over.  Returns the largest |E| sum seen
-// on a checked step (0 otherwise).
-template <typename T, bool CG>
+// on a checked step (0 otherwise).  PDL: the caller has not waited for the phase before; the first batch's
+// E and psi_E loads come first.
+template <typename T, bool CG, bool PDL = false>
 __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0, int k1, int n)
 {
     constexpr int P = kShellPZ;
@@ -688,14 +702,10 @@ __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0,
         const unsigned nx = (unsigned)p.nx, plane = (unsigned)p.plane, col = (unsigned)y * nx + (unsigned)x;
         const PsiCol pc = psi_col(p, x, y, sx, sy);
         const bool in_dxy = x >= p.db[0] && x < p.db[1] && y >= p.db[2] && y < p.db[3];
-        const T* __restrict__ H0 = p.Hn[0];
-        const T* __restrict__ H1 = p.Hn[1];
-        const T* __restrict__ H2 = p.Hn[2];
+        const T* H0 = p.Hn[0];
+        const T* H1 = p.Hn[1];
+        const T* H2 = p.Hn[2];
         T hxb = T(0), hyb = T(0);   // H_x, H_y of the plane below the batch
-        if (k0 > 0) {
-            hxb = ldf<CG>(H0 + (unsigned)(k0 - 1) * plane + col);
-            hyb = ldf<CG>(H1 + (unsigned)(k0 - 1) * plane + col);
-        }
         for (int kb = k0; kb < k1; kb += P) {   // (a compile-time trip bound here costs registers)
             T h[P][3], hm[P][4], e0[P][3], ps[P][6];
             bool on[P];
@@ -707,6 +717,26 @@ __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0,
                 on[r] = k < k1 && !(in_dxy && k >= p.db[4] && k < p.db[5]);
                 if (k >= k1) continue;
                 const unsigned id = (unsigned)k * plane + col;
+                e0[r][0] = ld_pre(p.E[0] + id);
+                e0[r][1] = ld_pre(p.E[1] + id);
+                e0[r][2] = ld_pre(p.E[2] + id);
+                psi_load(p.psiE, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
+            }
+            if (kb == k0) {
+                if (PDL) {
+                    pdl_wait();
+                    pdl_trigger();
+                }
+                if (k0 > 0) {
+                    hxb = ldf<CG>(H0 + (unsigned)(k0 - 1) * plane + col);
+                    hyb = ldf<CG>(H1 + (unsigned)(k0 - 1) * plane + col);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < P; ++r) {
+                const int k = kb + r;
+                if (k >= k1) continue;
+                const unsigned id = (unsigned)k * plane + col;
                 h[r][0] = ldf<CG>(H0 + id);
                 h[r][1] = ldf<CG>(H1 + id);
                 h[r][2] = ldf<CG>(H2 + id);
@@ -714,10 +744,6 @@ __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0,
                 hm[r][1] = y > 0 ? ldf<CG>(H0 + id - nx) : T(0);   // H_x(y-1)
                 hm[r][2] = x > 0 ? ldf<CG>(H2 + id - 1) : T(0);    // H_z(x-1)
                 hm[r][3] = x > 0 ? ldf<CG>(H1 + id - 1) : T(0);    // H_y(x-1)
-                e0[r][0] = ldf<CG>(p.E[0] + id);
-                e0[r][1] = ldf<CG>(p.E[1] + id);
-                e0[r][2] = ldf<CG>(p.E[2] + id);
-                psi_load<T, CG>(p.psiE, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
             }
 #pragma unroll
             for (int r = 0; r < P; ++r) {
@@ -777,21 +803,14 @@ __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0,
     return emax;
 }
 
-// E of the shell cells outside the design box.  It may run concurrently with the design-E kernel: the
-// last block of the two launches advances the step.
+// E of the shell cells outside the design box.  It may run concurrently with the design-E kernel.
 template <typename T>
 __global__ void __launch_bounds__(kBX * kBY, sizeof(T) == 8 ? 2 : FDTD_SHELL_MINB) shell_e_kernel(const KParams<T> p, const ShellBoxes s)
 {
-    pdl_wait();
-    pdl_trigger();
     ShellCol cl;
-    const bool live = shell_cell(s, cl);
-    const int n = read_step<T>(p.ctl);
-    if (live) {
-        const T emax = e_column<T, false>(p, cl.x, cl.y, cl.k0, cl.k1, n);
-        if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
-    }
-    finish_step(p.ctl, p.nblocks_e, n);
+    if (!shell_cell(s, cl)) return;
+    const T emax = e_column<T, false, true>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
+    if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
 }
 
 }  // namespace fdtd
