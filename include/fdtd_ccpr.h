@@ -130,9 +130,11 @@ typedef struct {
         bytes_dft_per_launch, bytes_grad_per_launch;
     double dft_steps_per_launch;             /* time steps folded into one DFT launch */
     long long fused_step;                    /* 1: the grid has an interior box for the fused TMA kernel
-                                                (x rows a multiple of 16 bytes, room inside the CPML);
+                                                (x rows a multiple of 16 bytes, room inside the CPML), which
+                                                takes it on large grids (see fdtd_set_step_layout);
                                                 0: the shell kernels cover the whole grid */
-    double interior_cells;                   /* cells of the interior box (one fused-kernel launch) */
+    double interior_cells;                   /* cells of one fused-kernel launch (0: the shell kernels take
+                                                the whole grid) */
     double interior_design_cells;            /* of which inside the working box (no E update there) */
     long long paired_shell;                  /* 1: the shell kernels update x-adjacent cell pairs (FP32, every
                                                 x bound of the grid, the x CPML and the shell boxes even) */
@@ -245,6 +247,12 @@ fdtd_status fdtd_get_gradient_constants(fdtd_handle h, double* dst, size_t n_dou
  * for other handles.  timeout_ns = 0 turns the hook off.  Errors: FDTD_ERR_ARG (a grid without an
  * interior box, where the step kernel does not run; timeout_ns outside [0, 1e10]). */
 fdtd_status fdtd_inject_wait_timeout(fdtd_handle h, long long timeout_ns);
+
+/* Which kernels take the background step: 0 (default) by grid size, 1 the shell kernels on the whole grid,
+ * 2 the interior kernel on its box and the shell kernels around it.  All give the same fields to the
+ * rounding of the build; the choice is a matter of speed.  Errors: FDTD_ERR_ARG (before fdtd_set_materials;
+ * other values; 2 on a grid without an interior box, see fdtd_timings.fused_step). */
+fdtd_status fdtd_set_step_layout(fdtd_handle h, int layout);
 
 /* Profiling: when on, runs time a sample of their kernel launches with CUDA events (see
  * fdtd_timings); fdtd_get_timings returns the sums since fdtd_reset_timings. */

@@ -22,7 +22,7 @@ EXPORTS = ("fdtd_create_grid", "fdtd_footprint_bytes", "fdtd_set_materials", "fd
            "fdtd_get_dft", "fdtd_get_index_map", "fdtd_set_profiling", "fdtd_get_timings",
            "fdtd_reset_timings", "fdtd_get_info", "fdtd_cancel", "fdtd_last_error", "fdtd_destroy",
            "fdtd_gradient_static", "fdtd_filter_project", "fdtd_filter_project_grad", "fdtd_paper_forward",
-           "fdtd_paper_gradient", "fdtd_get_gradient_constants", "fdtd_inject_wait_timeout", "fdtd_batch_create",
+           "fdtd_paper_gradient", "fdtd_get_gradient_constants", "fdtd_inject_wait_timeout", "fdtd_set_step_layout", "fdtd_batch_create",
            "fdtd_batch_submit", "fdtd_batch_run", "fdtd_batch_set_wait_limit", "fdtd_batch_set_blocks", "fdtd_batch_info",
            "fdtd_batch_destroy",
            "fdtd_get_objective")
@@ -103,6 +103,7 @@ def load_library():
         "fdtd_batch_destroy": [vp],
         "fdtd_get_objective": [vp, P(d), P(d)],
         "fdtd_inject_wait_timeout": [vp, C.c_longlong],
+        "fdtd_set_step_layout": [vp, i],
         "fdtd_get_index_map": [vp, i, P(C.c_int32), sz],
         "fdtd_set_profiling": [vp, i],
         "fdtd_get_timings": [vp, P(Timings)],
@@ -303,6 +304,10 @@ def fdtd_get_gradient_constants(h, n_freq):
 
 def fdtd_inject_wait_timeout(h, timeout_ns):
     _check(h, load_library().fdtd_inject_wait_timeout(h, int(timeout_ns)), "fdtd_inject_wait_timeout")
+
+
+def fdtd_set_step_layout(h, layout):
+    _check(h, load_library().fdtd_set_step_layout(h, int(layout)), "fdtd_set_step_layout")
 
 
 def fdtd_get_index_map(h, which, n):

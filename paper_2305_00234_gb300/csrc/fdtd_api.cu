@@ -47,6 +47,7 @@ const double kEps0 = 1.0 / (kMu0 * kC0 * kC0);
 const double kPi = 3.14159265358979323846;
 constexpr int kGraphSteps = fdtd::kMaxSnap;   // one DFT block per captured graph
 constexpr int kChunkSteps = 512;
+constexpr size_t kInteriorCells32 = 9000000, kInteriorCells64 = 300000;   // see Solver::interior
 constexpr int kProfEvery = 4;                  // profiling times one DFT block in four
 
 struct Err {
@@ -404,19 +405,25 @@ struct Solver : SolverBase {
     int* ctl = nullptr;
     int ptot[3] = {0, 0, 0};
     bool fused = false;             // an interior box for the fused TMA step kernel exists
+    int layout = 0;                 // fdtd_set_step_layout: 0 by size, 1 shell kernels only, 2 interior kernel
     bool use_pdl = true;            // step graphs with programmatic edges between phases (else captured)
     bool pdl_built = false;         // a step graph with programmatic edges has been instantiated
     StepMaps maps[2]{};             // tensor maps of the buffers read by even / odd steps
-    fdtd::ShellBoxes shell{};       // the cells around the interior box
+    fdtd::ShellBoxes shell_around{};   // the cells around the interior box
+    fdtd::ShellBoxes shell_all{};      // the whole grid
     std::vector<double2> ab_host;
     std::vector<double> gap_dft;     // host copy of the forward gap DFT, (f,c,gv) complex
     double adj_cond = 0.0;
     cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [mode][full, remainder]
 
     explicit Solver(fdtd_ctx* ctx) : c(ctx) {}
-    void interior_box(int ib[6]) const override { std::copy(base.ib, base.ib + 6, ib); }
+    void interior_box(int ib[6]) const override
+    {
+        if (interior()) std::copy(base.ib, base.ib + 6, ib);
+        else std::fill(ib, ib + 6, 0);
+    }
     bool has_interior() const override { return fused; }
-    bool paired_shell() const override { return shell.pair != 0; }
+    bool paired_shell() const override { return shell().pair != 0; }
     bool pdl_graphs() const override { return use_pdl && pdl_built; }
     bool paired_design() const override { return base.ed_pair != 0; }
     ~Solver() override
@@ -424,6 +431,27 @@ struct Solver : SolverBase {
         for (auto& g : graph)
             for (auto& x : g)
                 if (x) cudaGraphExecDestroy(x);
+    }
+
+    // Whether the interior box is the fused kernel's, or the shell kernels take the whole grid, as they do on
+    // grids below kInteriorCells32 / 64 cells: the fused kernel moves a third fewer bytes, but a block of it
+    // is a chain of TMA latency, plane by plane, that a small launch cannot hide, while much of such a grid
+    // stays in L2.  Measured, one step with / without the fused kernel (FP32, three poles, 8-cell CPML): 64^3
+    // 18 / 12 us, 128^3 50 / 42, 160^3 85 / 76, 192^3 127 / 125, 128 x 256 x 256 158 / 151, 208^3 157 / 159, 224^3
+    // 193 / 195, 256^3 267 / 283.  FP64: 52 x 48 x 44 59 / 47, 64^3 90 / 89, 96^3 209 / 239.
+    // An armed wait-timeout hook asks for the fused kernel's wait.
+    bool interior() const
+    {
+        if (!fused || layout == 1) return false;
+        return layout == 2 || base.stall_ns > 0 || c->ncell >= (sizeof(T) == 4 ? kInteriorCells32 : kInteriorCells64);
+    }
+    const fdtd::ShellBoxes& shell() const { return interior() ? shell_around : shell_all; }
+
+    void set_layout(int l)
+    {
+        if (l == 2 && !fused) arg_error("step layout 2 needs a grid with an interior box");
+        layout = l;
+        refresh_params();
     }
 
     T* talloc(size_t n) { return (T*)c->alloc(n * sizeof(T)); }
@@ -558,8 +586,10 @@ struct Solver : SolverBase {
         CK(cudaMemsetAsync(ctl, 0, 4 * sizeof(int), c->work));
         p.ctl = ctl;
         for (int m = 0; m < 2; ++m) dp[m].ctl = ctl;
-        shell.pair = shell_pairable(p) ? 1 : 0;
-        fdtd::shell_blocks(shell);
+        for (fdtd::ShellBoxes* b : {&shell_around, &shell_all}) {
+            b->pair = shell_pairable(p, *b) ? 1 : 0;
+            fdtd::shell_shape(*b, (int)sizeof(T));
+        }
         p.edz = 1;
         p.ed_pair = design_pairable() ? 1 : 0;
         if (c->nd) p.edz = fdtd::design_planes((p.ed_pair ? c->dn[0] / 2 : c->dn[0]) * c->dn[1], c->dn[2]);
@@ -762,7 +792,11 @@ struct Solver : SolverBase {
     }
 
     // Interior box of the fused kernel: kTX x kTY tiles whose cells and one-cell -x/-y halo lie outside
-    // the walls and the CPML slabs, x0 a multiple of 4 (16-byte aligned TMA boxes), planes cpml_z_low + 1
+    // the walls and the CPML slabs, x0 a multiple of 32 bytes, or of 128 where the x rows are (whole sectors,
+    // or whole lines, in every tile row's stores: with x0 at 48 or 80 bytes from a line the kernel wrote half
+    // sectors that two tiles share, and ran at 4.7 TB/s instead of 6.2 on a 512 x 512 x 384 grid, a step of
+    // which went from 1909 to 1658 us; 256^3 with a 12-cell CPML, x0 at 64 and at 128 bytes: 275 and 271 us;
+    // 208^3, whose rows are no multiple of 128 bytes, x0 at 64 and at 128 bytes: 157 and 165 us), planes cpml_z_low + 1
     // .. nz - cpml_z_high - 1 (the plane below the first one is outside the slab too), at least one whole
     // tile each way.  Toward the +x and +y slabs the box ends in a partial tile column or row (an even
     // number of x cells; the kernel leaves the cells beyond to the shell) when that tile holds at least
@@ -784,7 +818,14 @@ struct Solver : SolverBase {
     void split_grid(KParams<T>& p)
     {
         const fdtd_grid_desc& d = c->d;
-        const int X0 = (std::max(p.cpl[0] + 1, 1) + 3) / 4 * 4, Y0 = std::max(p.cpl[1] + 1, 1), Z0 = p.cpl[2] + 1;
+        int X0 = 0;
+        for (int line : {128, 32, 16}) {   // the largest alignment that leaves room for a tile
+            const int xa = line / (int)sizeof(T);
+            if (line == 128 && d.nx % xa) continue;
+            X0 = std::max((std::max(p.cpl[0] + 1, 1) + xa - 1) / xa * xa, 4);
+            if (d.nx - p.cph[0] - X0 >= fdtd::kTX) break;
+        }
+        const int Y0 = std::max(p.cpl[1] + 1, 1), Z0 = p.cpl[2] + 1;
         const int wx = d.nx - p.cph[0] - X0, wy = d.ny - p.cph[1] - Y0;   // widths up to the +x / +y slabs
         const int Z1 = d.nz - p.cph[2];
         fused = ((size_t)d.nx * sizeof(T)) % 16 == 0 && wx >= fdtd::kTX && wy >= fdtd::kTY && Z1 > Z0 &&
@@ -800,28 +841,26 @@ struct Solver : SolverBase {
         p.kc = fdtd::kKC;
         if (fused)
             while (p.kc > 2 && (unsigned)ntx * nty * ((Z1 - Z0 + p.kc - 1) / p.kc) < FDTD_STEP_MINBLK) p.kc /= 2;
-        shell = fdtd::ShellBoxes{};
-        auto add = [&](int x0, int x1, int y0, int y1, int z0, int z1) {
+        auto add = [](fdtd::ShellBoxes& s, int x0, int x1, int y0, int y1, int z0, int z1) {
             if (x0 >= x1 || y0 >= y1 || z0 >= z1) return;
-            int* b = shell.b[shell.n++];
+            int* b = s.b[s.n++];
             b[0] = x0; b[1] = x1; b[2] = y0; b[3] = y1; b[4] = z0; b[5] = z1;
         };
-        if (!fused) {
-            add(0, d.nx, 0, d.ny, 0, d.nz);
-        } else {
-            add(0, d.nx, 0, d.ny, 0, ib[4]);                      // below and above the interior planes
-            add(0, d.nx, 0, d.ny, ib[5], d.nz);
-            add(0, d.nx, 0, ib[2], ib[4], ib[5]);                 // in front of and behind it in y
-            add(0, d.nx, ib[3], d.ny, ib[4], ib[5]);
-            add(0, ib[0], ib[2], ib[3], ib[4], ib[5]);            // left and right of it in x
-            add(ib[1], d.nx, ib[2], ib[3], ib[4], ib[5]);
-        }
+        add(shell_all, 0, d.nx, 0, d.ny, 0, d.nz);
+        if (!fused) return;
+        fdtd::ShellBoxes& s = shell_around;
+        add(s, 0, d.nx, 0, d.ny, 0, ib[4]);                       // below and above the interior planes
+        add(s, 0, d.nx, 0, d.ny, ib[5], d.nz);
+        add(s, 0, d.nx, 0, ib[2], ib[4], ib[5]);                  // in front of and behind it in y
+        add(s, 0, d.nx, ib[3], d.ny, ib[4], ib[5]);
+        add(s, 0, ib[0], ib[2], ib[3], ib[4], ib[5]);             // left and right of it in x
+        add(s, ib[1], d.nx, ib[2], ib[3], ib[4], ib[5]);
     }
 
     // The paired shell kernels (FP32) need the x boundaries of the grid, of the CPML slabs and of the
     // shell boxes even (the two cells of a pair on the same side of each); the working box's x bounds,
     // the TF/SF plane and point sources may fall between the cells of a pair.
-    bool shell_pairable(const KParams<T>& p) const
+    bool shell_pairable(const KParams<T>& p, const fdtd::ShellBoxes& shell) const
     {
         if (sizeof(T) != 4 || p.nx % 2 || p.cpl[0] % 2 || p.cph[0] % 2) return false;
         for (int q = 0; q < shell.n; ++q)
@@ -851,18 +890,18 @@ struct Solver : SolverBase {
     {
         if (!mp) mp = maps;
         cudaError_t e = cudaSuccess;
-        if (concurrent && fused) {
+        if (concurrent && interior()) {
             e = cudaEventRecord(c->fork, c->work);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->fork, 0);
-            if (e == cudaSuccess) e = fdtd::launch_shell<T>(q, shell, false, c->side);
+            if (e == cudaSuccess) e = fdtd::launch_shell<T>(q, shell(), false, c->side);
             if (e == cudaSuccess) e = fdtd::launch_step<T>(q, mp[parity & 1], c->work);
             if (e == cudaSuccess) e = cudaEventRecord(c->join, c->side);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(c->work, c->join, 0);
         } else {
-            e = fdtd::launch_shell<T>(q, shell, false, c->work);
-            if (e == cudaSuccess && fused) e = fdtd::launch_step<T>(q, mp[parity & 1], c->work);
+            e = fdtd::launch_shell<T>(q, shell(), false, c->work);
+            if (e == cudaSuccess && interior()) e = fdtd::launch_step<T>(q, mp[parity & 1], c->work);
         }
-        return e == cudaSuccess ? fdtd::launch_shell<T>(q, shell, true, c->work) : e;
+        return e == cudaSuccess ? fdtd::launch_shell<T>(q, shell(), true, c->work) : e;
     }
 
     // One whole time step: the H phase (shell H next to the interior kernel when concurrent), then
@@ -877,13 +916,13 @@ struct Solver : SolverBase {
         if (!mp) mp = maps;
         cudaError_t e = cudaEventRecord(c->fork, c->work);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->fork, 0);
-        if (e == cudaSuccess) e = fdtd::launch_shell<T>(q, shell, false, c->side);
-        if (e == cudaSuccess && fused) e = fdtd::launch_step<T>(q, mp[parity & 1], c->work);
+        if (e == cudaSuccess) e = fdtd::launch_shell<T>(q, shell(), false, c->side);
+        if (e == cudaSuccess && interior()) e = fdtd::launch_step<T>(q, mp[parity & 1], c->work);
         if (e == cudaSuccess) e = cudaEventRecord(c->join, c->side);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(c->work, c->join, 0);
         if (e == cudaSuccess) e = cudaEventRecord(c->fork, c->work);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->fork, 0);
-        if (e == cudaSuccess) e = fdtd::launch_shell<T>(q, shell, true, c->side);
+        if (e == cudaSuccess) e = fdtd::launch_shell<T>(q, shell(), true, c->side);
         if (e == cudaSuccess) e = fdtd::launch_e_design<T>(q, htab, bucket, c->work);
         if (e == cudaSuccess) e = cudaEventRecord(c->join, c->side);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(c->work, c->join, 0);
@@ -1065,7 +1104,7 @@ struct Solver : SolverBase {
             CK(launch_one_step(q, s, true, mp));   // both phases on two streams, as in the captured graphs
         }
         if (n_to > n_from) CK(fdtd::launch_block_end(p.ctl, n_to - n_from, c->work));
-        c->tim.launches += (long long)(n_to - n_from) * (fused ? 4 : 3);
+        c->tim.launches += (long long)(n_to - n_from) * (interior() ? 4 : 3);
     }
 
     void pm_check(const int* ctl_dev, int expect)
@@ -1269,7 +1308,7 @@ struct Solver : SolverBase {
             cudaGetLastError();
             return nullptr;
         }
-        const bool has_shell = shell.first[shell.n] > 0;   // the fused kernel may cover the whole grid
+        const bool has_shell = shell().first[shell().n] > 0;   // the fused kernel may cover the whole grid
         cudaGraphEdgeData ed = {};
         ed.type = cudaGraphDependencyTypeProgrammatic;
         ed.from_port = cudaGraphKernelNodePortProgrammatic;
@@ -1289,13 +1328,13 @@ struct Solver : SolverBase {
             const KParams<T> q = par(p, st, st);
             phase([&] {
                 cudaGraphNode_t n = nullptr;
-                if (e == cudaSuccess && has_shell && (e = fdtd::graph_shell<T>(g, &n, q, shell, false)) == cudaSuccess)
+                if (e == cudaSuccess && has_shell && (e = fdtd::graph_shell<T>(g, &n, q, shell(), false)) == cudaSuccess)
                     cur.push_back(n);
-                if (e == cudaSuccess && fused && (e = fdtd::graph_step<T>(g, &n, q, maps[st & 1])) == cudaSuccess) cur.push_back(n);
+                if (e == cudaSuccess && interior() && (e = fdtd::graph_step<T>(g, &n, q, maps[st & 1])) == cudaSuccess) cur.push_back(n);
             });
             phase([&] {
                 cudaGraphNode_t n = nullptr;
-                if (e == cudaSuccess && has_shell && (e = fdtd::graph_shell<T>(g, &n, q, shell, true)) == cudaSuccess)
+                if (e == cudaSuccess && has_shell && (e = fdtd::graph_shell<T>(g, &n, q, shell(), true)) == cudaSuccess)
                     cur.push_back(n);
                 if (e == cudaSuccess && c->nd && (e = fdtd::graph_e_design<T>(g, &n, q, htab, bucket)) == cudaSuccess)
                     cur.push_back(n);
@@ -1392,11 +1431,11 @@ struct Solver : SolverBase {
                     const KParams<T> pp = par(p, s, q);
                     cudaEvent_t* e = &c->ev[5 * (size_t)s];
                     CK(cudaEventRecord(e[0], c->work));
-                    CK(fdtd::launch_shell<T>(pp, shell, false, c->work));
+                    CK(fdtd::launch_shell<T>(pp, shell(), false, c->work));
                     CK(cudaEventRecord(e[1], c->work));
-                    if (fused) CK(fdtd::launch_step<T>(pp, maps[s & 1], c->work));
+                    if (interior()) CK(fdtd::launch_step<T>(pp, maps[s & 1], c->work));
                     CK(cudaEventRecord(e[2], c->work));
-                    CK(fdtd::launch_shell<T>(pp, shell, true, c->work));
+                    CK(fdtd::launch_shell<T>(pp, shell(), true, c->work));
                     CK(cudaEventRecord(e[3], c->work));
                     CK(fdtd::launch_e_design<T>(pp, htab, bucket, c->work));
                     CK(cudaEventRecord(e[4], c->work));
@@ -1430,13 +1469,13 @@ struct Solver : SolverBase {
         }
         c->tim.shell_h_launches += timed_steps;    // launches that were timed (profiling samples)
         c->tim.shell_e_launches += timed_steps;
-        if (fused) c->tim.step_launches += timed_steps;
+        if (interior()) c->tim.step_launches += timed_steps;
         if (c->nd) c->tim.ed_launches += timed_steps;
         if (c->nd) {
             c->tim.dft_launches += timed_blocks;
             c->tim.launches += nblk;
         }
-        c->tim.launches += ((fused ? 3LL : 2LL) + (c->nd ? 1LL : 0LL)) * M;  // every kernel this run launched
+        c->tim.launches += ((interior() ? 3LL : 2LL) + (c->nd ? 1LL : 0LL)) * M;  // every kernel this run launched
         c->tim.fused_step = fused ? 1 : 0;
         int hctl[4];
         CK(cudaMemcpyAsync(hctl, ctl, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->work));
@@ -2469,6 +2508,16 @@ fdtd_status fdtd_inject_wait_timeout(fdtd_handle h, long long timeout_ns)
         return FDTD_ERR_ARG;
     }
     return guarded(h, [&] { dispatch(h, [&](auto* s) { s->set_stall(timeout_ns); }); });
+}
+
+fdtd_status fdtd_set_step_layout(fdtd_handle h, int layout)
+{
+    if (fdtd_status s = check_handle(h)) return s;
+    if (!h->impl || layout < 0 || layout > 2) {
+        h->err = "step layout must be 0 (by size), 1 (shell kernels) or 2 (interior kernel), after set_materials";
+        return FDTD_ERR_ARG;
+    }
+    return guarded(h, [&] { dispatch(h, [&](auto* s) { s->set_layout(layout); }); });
 }
 
 fdtd_status fdtd_get_index_map(fdtd_handle h, int which, int32_t* dst, size_t n)

@@ -24,7 +24,7 @@ constexpr int kMaxSnap = 16;      // steps per blocked DFT update (snapshot ring
 #define FDTD_KC 8
 #endif
 #ifndef FDTD_SHELL_KZ
-#define FDTD_SHELL_KZ 8
+#define FDTD_SHELL_KZ 16
 #endif
 #ifndef FDTD_ED_Z
 #define FDTD_ED_Z 8
@@ -91,6 +91,7 @@ struct ShellBoxes {
     int b[6][6];          // half-open x0, x1, y0, y1, z0, z1
     unsigned first[7];
     int kz;               // z planes per thread (<= kShellKZ)
+    int nt;               // threads per block (a multiple of kBX)
     int pair;             // 1: the paired kernels (a thread per two x-adjacent columns; every x bound even)
 };
 

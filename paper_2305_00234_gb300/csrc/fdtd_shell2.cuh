@@ -50,9 +50,9 @@ __device__ __forceinline__ bool shell_pair(const ShellBoxes& s, ShellCol& c)
     const int* B = s.b[q];
     const unsigned loc = blockIdx.x - s.first[q];
     const unsigned wx = (unsigned)(B[1] - B[0]) / 2u, wxy = wx * (B[3] - B[2]);
-    const unsigned chunks = (wxy + kShellCells - 1) / kShellCells;
+    const unsigned chunks = (wxy + s.nt - 1) / s.nt;
     const unsigned zc = loc / chunks;
-    const unsigned t = (loc - zc * chunks) * kShellCells + threadIdx.y * kBX + threadIdx.x;
+    const unsigned t = (loc - zc * chunks) * s.nt + threadIdx.y * kBX + threadIdx.x;
     const unsigned yy = t / wx;
     c.x = B[0] + 2 * (int)(t - yy * wx);
     c.y = B[2] + (int)yy;
@@ -138,9 +138,8 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_h2_kernel(c
     const float* E2 = p.E[2];
     const float2 z2 = f2(0.f, 0.f);
     float2 exc, eyc;
-    for (int it = 0; it < kShellKZ / P; ++it) {
-        const int kb = cl.k0 + it * P;
-        if (kb >= cl.k1) break;
+    for (int kb = cl.k0; kb < cl.k1; kb += P) {
+        const int it = kb - cl.k0;
         float2 ex0[P], ey0[P], ez0[P], ezy[P], exy[P], ezx[P], eyx[P], exz[P], eyz[P], ho[P][3], ps[P][6];
         int sz[P];
 #pragma unroll

@@ -480,14 +480,12 @@ __global__ void __launch_bounds__(kPX * kTY, StepCfg<T>::MINB)
 }
 
 // ---- shell: per-cell kernels ----------------------------------------------------------------------
-// Block b -> box q; a block covers kShellCells consecutive (x, y) columns of the box (x fastest, so a
+// Block b -> box q; a block covers s.nt consecutive (x, y) columns of the box (x fastest, so a
 // warp reads and writes consecutive addresses even in boxes narrower than a warp), and each thread
 // marches s.kz (at most kShellKZ) planes of its column in batches of kShellPZ planes whose loads are all
 // issued before any store.  The per-column set-up (box search, column coordinates, slab indices) is
 // paid once per s.kz planes; cell and psi offsets are 32-bit (a grid holds fewer than 2^31
 // cells) and advance by a fixed stride per plane.
-constexpr int kShellCells = kBX * kBY;
-
 struct ShellCol {
     int x, y, k0, k1;   // column, planes [k0, k1)
 };
@@ -499,9 +497,9 @@ __device__ __forceinline__ bool shell_cell(const ShellBoxes& s, ShellCol& c)
     const int* B = s.b[q];
     const unsigned loc = blockIdx.x - s.first[q];
     const unsigned wx = B[1] - B[0], wxy = wx * (B[3] - B[2]);
-    const unsigned chunks = (wxy + kShellCells - 1) / kShellCells;
+    const unsigned chunks = (wxy + s.nt - 1) / s.nt;
     const unsigned zc = loc / chunks;
-    const unsigned t = (loc - zc * chunks) * kShellCells + threadIdx.y * kBX + threadIdx.x;
+    const unsigned t = (loc - zc * chunks) * s.nt + threadIdx.y * kBX + threadIdx.x;
     const unsigned yy = t / wx;
     c.x = B[0] + (int)(t - yy * wx);
     c.y = B[2] + (int)yy;

@@ -139,6 +139,10 @@ class Problem:
         """Failure-path test hook (fdtd_inject_wait_timeout)."""
         N.fdtd_inject_wait_timeout(self.h, timeout_ns)
 
+    def set_step_layout(self, layout):
+        """0 by grid size (default), 1 shell kernels only, 2 interior kernel (fdtd_set_step_layout)."""
+        N.fdtd_set_step_layout(self.h, layout)
+
     def index_map(self, which):
         shape = ((3,) + self.n) if which <= 1 else self.n
         return N.fdtd_get_index_map(self.h, which, int(np.prod(shape))).reshape(shape)
