@@ -47,7 +47,7 @@ const double kEps0 = 1.0 / (kMu0 * kC0 * kC0);
 const double kPi = 3.14159265358979323846;
 constexpr int kGraphSteps = fdtd::kMaxSnap;   // one DFT block per captured graph
 constexpr int kChunkSteps = 512;
-constexpr size_t kInteriorCells32 = 9000000, kInteriorCells64 = 300000;   // see Solver::interior
+constexpr size_t kInteriorCells32 = 9000000, kInteriorCells64 = 600000;   // see Solver::interior
 constexpr int kProfEvery = 4;                  // profiling times one DFT block in four
 
 struct Err {
@@ -438,7 +438,7 @@ struct Solver : SolverBase {
     // is a chain of TMA latency, plane by plane, that a small launch cannot hide, while much of such a grid
     // stays in L2.  Measured, one step with / without the fused kernel (FP32, three poles, 8-cell CPML): 64^3
     // 18 / 12 us, 128^3 50 / 42, 160^3 85 / 76, 192^3 127 / 125, 128 x 256 x 256 158 / 151, 208^3 157 / 159, 224^3
-    // 193 / 195, 256^3 267 / 283.  FP64: 52 x 48 x 44 59 / 47, 64^3 90 / 89, 96^3 209 / 239.
+    // 193 / 195, 256^3 267 / 283.  FP64: 64^3 79 / 65, 80^3 106 / 104, 96^3 169 / 176.
     // An armed wait-timeout hook asks for the fused kernel's wait.
     bool interior() const
     {

