@@ -407,6 +407,25 @@ cudaError_t launch_paper_grad(const PParams<T>& g, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// Gradient sums times the cell volume, in the caller's type.
+template <typename O>
+__global__ void paper_scale_kernel(const double* __restrict__ g, double dV, long long n, O* __restrict__ out)
+{
+    const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v < n) out[v] = (O)(g[v] * dV);
+}
+
+cudaError_t launch_paper_scale(const double* g, double dV, long long n, void* out, int dtype, cudaStream_t s)
+{
+    if (n == 0) return cudaSuccess;
+    const unsigned nb = (unsigned)((n + 255) / 256);
+    if (dtype == 1)
+        paper_scale_kernel<double><<<nb, 256, 0, s>>>(g, dV, n, (double*)out);
+    else
+        paper_scale_kernel<float><<<nb, 256, 0, s>>>(g, dV, n, (float*)out);
+    return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_rho_scatter(const void* src, int dtype, long long n, const long long off[4], const int md[3][3],
                                int dnx, int dny, long long nd, T* dst, int* flag, cudaStream_t s)

@@ -52,6 +52,7 @@ template <typename T>
 cudaError_t launch_paper_drive(const T* gh, T* drive, int M, int ns, double eps0, cudaStream_t s);
 template <typename T>
 cudaError_t launch_paper_grad(const PParams<T>& g, cudaStream_t s);
+cudaError_t launch_paper_scale(const double* g, double dV, long long n, void* out, int dtype, cudaStream_t s);
 template <typename T>
 cudaError_t launch_index_map(const KParams<T>& p, int which, int32_t* out, cudaStream_t s);
 // persistent batch kernel (fdtd_batch.cu): its function for a pole bucket, and resident blocks per SM
