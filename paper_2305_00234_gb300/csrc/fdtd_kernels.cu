@@ -1,4 +1,5 @@
 // Launch wrappers and helper kernels; explicit FP32 / FP64 instantiations.
+#include <mutex>
 #include <utility>
 
 #include "fdtd_design2.cuh"
@@ -112,12 +113,19 @@ int pole_bucket(int max_poles)
     return max_poles == 0 ? 0 : max_poles <= 4 ? 4 : max_poles <= 8 ? 8 : 16;
 }
 
+// Dynamic shared memory limits of the kernels that need them raised, once per device and type.
 template <typename T>
-cudaError_t prepare_step()
+cudaError_t prepare_step(int device)
 {
-    const cudaError_t e = cudaFuncSetAttribute(dft_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DftSmem<T>::total);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(step_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)StepSmem<T>::total);
+    static std::mutex mutex;
+    static unsigned long long done = 0;   // bit per device (ordinals below 64)
+    std::lock_guard<std::mutex> lock(mutex);
+    if (done >> device & 1) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(dft_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DftSmem<T>::total);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(step_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)StepSmem<T>::total);
+    if (e == cudaSuccess) done |= 1ull << device;
+    return e;
 }
 
 // A kernel node of a step graph (no dependencies yet; the host adds them).
@@ -442,7 +450,7 @@ cudaError_t launch_rho_scatter(const void* src, int dtype, long long n, const lo
 }
 
 #define FDTD_INSTANTIATE(T)                                                                              \
-    template cudaError_t prepare_step<T>();                                                              \
+    template cudaError_t prepare_step<T>(int);                                                           \
     template cudaError_t graph_step<T>(cudaGraph_t, cudaGraphNode_t*, const KParams<T>&, const StepMaps&); \
     template cudaError_t graph_shell<T>(cudaGraph_t, cudaGraphNode_t*, const KParams<T>&, const ShellBoxes&, bool); \
     template cudaError_t graph_e_design<T>(cudaGraph_t, cudaGraphNode_t*, const KParams<T>&, const PoleTable<T>&, int); \

@@ -9,7 +9,7 @@ namespace fdtd {
 
 int pole_bucket(int max_poles);
 template <typename T>
-cudaError_t prepare_step();
+cudaError_t prepare_step(int device);
 // pdl: launch as a programmatic dependent launch in the step chain (see pdl_wait in fdtd_kernels.cuh)
 // kernel nodes of a step graph, without dependencies
 template <typename T>
