@@ -230,20 +230,19 @@ cudaError_t launch_step(const KParams<T>& p, const StepMaps& m, cudaStream_t s, 
     return launch_chain(step_kernel<T>, g, dim3(kPX, kTY), StepSmem<T>::total, s, pdl, p, m);
 }
 
-// Shape of the shell launches: z planes per thread and threads per block, by an estimate of the busiest SM's
-// time.  A column is a serial chain: with c blocks resident a plane (FP32 one-cell kernels: a batch of
-// planes; FP64: its arithmetic's latency) waits L and a plane takes c t of the SM; an SM runs its b blocks C at a time, and every
-// block costs the launch g.  L, t, g (us, t for 256 threads) and C are read off steps of 48^3 to 192^3 grids
-// and of 96 x 170 x 170 with every depth from 1 to 16.  What it decides: one full round of long columns instead of
-// one and a little (96 x 170 x 170: depth 9, 608 blocks, a step 60 us; depth 8, 704 blocks, 68; 128^3: depths 7 to
-// 9 42 us, 6 47), and short columns, in blocks that spread evenly, where a grid has few of them (48^3: depth 1
-// in blocks of 128 9.4 us, 4 in blocks of 256 12.9).  Past three rounds only L/C + t a plane matters, which
-// the depth does not change, and it stays at kLongColumn.
+// Shape of the shell launches: z planes per thread and threads per block, by an estimate of the busiest SM's time.
+// A column is a serial chain: with c blocks resident a plane (FP64: its arithmetic's latency) waits L and a plane
+// takes c t of the SM; an SM runs its b blocks C at a time, and every block costs the launch g.  L, t, g (us, t for
+// 256 threads) and C are read off steps of 48^3 to 192^3 grids and of 96 x 170 x 170 with every depth from 1 to 16.
+// What it decides: one full round of long columns instead of one and a little (96 x 170 x 170: depth 9, 608 blocks,
+// a step 60 us; depth 8, 704 blocks, 68; 128^3: depths 7 to 9 42 us, 6 47), and short columns, in blocks that spread
+// evenly, where a grid has few of them (48^3: depth 1 in blocks of 128 9.4 us, 4 in blocks of 256 12.9).  Past three
+// rounds only L/C + t a plane matters, which the depth does not change, and it stays at kLongColumn.
 void shell_shape(ShellBoxes& s, int type_bytes)
 {
     const bool f64 = type_bytes == 8;
     const double L = f64 ? 1.2 : 0.7, t256 = f64 ? 3.3 : (s.pair ? 0.45 : 0.25), g = 0.003;
-    const int batch = s.pair || f64 ? 1 : kShellPZ, resident256 = f64 ? 2 : 4, sms = 152;
+    const int resident256 = f64 ? 2 : 4, sms = 152;
     auto blocks = [&](int kz, int nt) {
         unsigned t = 0;
         for (int q = 0; q < s.n; ++q) {
@@ -264,7 +263,7 @@ void shell_shape(ShellBoxes& s, int type_bytes)
             const unsigned C = resident256 * 256 / nt;
             if (kz > kLongColumn && b > 3 * C) continue;
             // FP32 blocks of 128 threads find fewer of their neighbours' rows in L1
-            const double t = t256 * nt / 256.0 * (nt < 256 && !f64 ? 1.05 : 1.0), wait = (kz + batch - 1) / batch * L;
+            const double t = t256 * nt / 256.0 * (nt < 256 && !f64 ? 1.05 : 1.0), wait = kz * L;
             const double cost = (b / C) * (wait + kz * C * t) + (b % C ? wait + kz * (b % C) * t : 0.0) + g * nb;
             if (s.kz == 0 || cost < best) {
                 best = cost;

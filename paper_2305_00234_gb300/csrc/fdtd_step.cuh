@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(kPX * kTY, StepCfg<T>::MINB)
 // ---- shell: per-cell kernels ----------------------------------------------------------------------
 // Block b -> box q; a block covers s.nt consecutive (x, y) columns of the box (x fastest, so a
 // warp reads and writes consecutive addresses even in boxes narrower than a warp), and each thread
-// marches s.kz (at most kShellKZ) planes of its column in batches of kShellPZ planes whose loads are all
+// marches s.kz (at most kShellKZ) planes of its column in batches of kShellPZ<T> planes whose loads are all
 // issued before any store.  The per-column set-up (box search, column coordinates, slab indices) is
 // paid once per s.kz planes; cell and psi offsets are 32-bit (a grid holds fewer than 2^31
 // cells) and advance by a fixed stride per plane.
@@ -595,7 +595,7 @@ __device__ __forceinline__ T stretch_v(T d, const T* __restrict__ tab, int s, T&
 template <typename T, bool CG, bool PDL = false>
 __device__ __forceinline__ void h_column(const KParams<T>& p, int x, int y, int k0, int k1, int n)
 {
-    constexpr int P = kShellPZ;
+    constexpr int P = kShellPZ<T>;
     const T cneg = -(p.ch * p.inv_dx), idx = p.inv_dx, ch = p.ch;
     const T einc_n = p.tfsf_i0 >= 0 ? __ldg(p.einc + n) : T(0);
     const bool tf = x == p.tfsf_i0 - 1;   // H_y here is scattered field
@@ -724,7 +724,7 @@ __global__ void __launch_bounds__(kBX * kBY, sizeof(T) == 8 ? 2 : FDTD_SHELL_MIN
 template <typename T, bool CG, bool PDL = false>
 __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0, int k1, int n)
 {
-    constexpr int P = kShellPZ;
+    constexpr int P = kShellPZ<T>;
     T emax = T(0);
     {
         const T hinc_n = p.tfsf_i0 >= 0 ? __ldg(p.hinc + n) : T(0);
