@@ -2,9 +2,9 @@
 // (Maxwells)a,b with (eps_mixed), (sigma_mixed), (Poles_mixed) and the pole recursion, as in
 // e_design_column, with each thread updating the samples of component C at (i, j, k) and (i+1, j, k):
 // 8-byte loads and stores of fields, densities and snapshots, 16-byte loads and stores of the two
-// samples' pole currents, and Blackwell's paired FP32 instructions.  Pairs that need a per-sample
-// treatment (a gap sample, a point source, the TF/SF plane, a PEC wall, a sample outside its
-// component's sample box) and the per-sample records of paper mode take e_design_column sample by sample.
+// samples' pole currents, and Blackwell's paired FP32 instructions.  Samples outside their component's sample
+// box or in the gap, point sources and the TF/SF plane are handled within the pair; pairs on a PEC wall and the
+// per-sample records of paper mode take e_design_column sample by sample.
 //
 // Used when nx and the working box's x origin and extent are even (the host checks), so that a pair's two
 // samples are adjacent, and 8-byte aligned, in every array (the density too, in either layout).
@@ -34,12 +34,12 @@ __device__ __forceinline__ float design_pair_column(const KParams<float>& p, con
     const float* rc = p.rhoc[C];
     const unsigned nx = (unsigned)p.nx, plane = (unsigned)p.plane, col = (unsigned)j * nx + (unsigned)i;
     const long long dcol = (long long)(j - p.db[2]) * p.dnx + (i - p.db[0]);
-    const bool inxy_g = i + 1 >= p.gb[0] && i < p.gb[1] && j >= p.gb[2] && j < p.gb[3];   // either sample
-    // per-sample cases for the whole column: paper-mode records, either sample outside the component's
-    // sample box in x or y, the TF/SF plane (E_z at x = i0), the PEC walls at x = 0 (C = 1, 2), y = 0 (C = 0, 2)
-    const bool col_scalar = p.td_acc || p.hist_dq || i < p.mb[C][0] || i + 1 >= p.mb[C][1] || j < p.mb[C][2] ||
-                            j >= p.mb[C][3] || (C == 2 && (i == p.tfsf_i0 || i + 1 == p.tfsf_i0)) ||
-                            ((C == 1 || C == 2) && i == 0) || (C != 1 && j == 0);
+    // which of the two samples lie in the component's sample box and in the gap box, in x and y
+    const bool iny = j >= p.mb[C][2] && j < p.mb[C][3], gy = j >= p.gb[2] && j < p.gb[3];
+    const bool m0 = iny && i >= p.mb[C][0] && i < p.mb[C][1], m1 = iny && i + 1 >= p.mb[C][0] && i + 1 < p.mb[C][1];
+    const bool g0 = gy && i >= p.gb[0] && i < p.gb[1], g1 = gy && i + 1 >= p.gb[0] && i + 1 < p.gb[1];
+    // per-sample cases for the whole column: paper-mode records, the PEC walls at x = 0 (C = 1, 2), y = 0 (C = 0, 2)
+    const bool col_scalar = p.td_acc || p.hist_dq || ((C == 1 || C == 2) && i == 0) || (C != 1 && j == 0);
     const long long slot0 = (long long)((n - p.snap0) % p.K) * p.snap_stride + C * p.nd;
     const int P = p.P[C], P1 = p.P1[C];
     const float2 idx2 = f2(p.inv_dx, p.inv_dx), one2 = f2(1.f, 1.f);
@@ -50,9 +50,8 @@ __device__ __forceinline__ float design_pair_column(const KParams<float>& p, con
         const bool in_gz = k >= p.gb[4] && k < p.gb[5];
         const bool src = p.nb > 0 && k >= p.sb[4] && k < p.sb[5] && j >= p.sb[2] && j < p.sb[3] && i + 1 >= p.sb[0] &&
                          i < p.sb[1];
-        // per-sample cases of this plane: a gap sample, a point source, the z range of the sample box, the
-        // PEC wall at z = 0 (C = 0, 1)
-        if (col_scalar || src || (in_gz && inxy_g) || k < p.mb[C][4] || k >= p.mb[C][5] || (C != 2 && k == 0)) {
+        // per-sample cases of this plane: the PEC wall at z = 0 (C = 0, 1)
+        if (col_scalar || (C != 2 && k == 0)) {
             pdl_wait();   // (returns at once when the phase before is complete)
             pdl_trigger();
 #pragma unroll 1
@@ -61,6 +60,10 @@ __device__ __forceinline__ float design_pair_column(const KParams<float>& p, con
         }
         const unsigned id = (unsigned)k * plane + col;
         const long long dv = (long long)(k - p.db[4]) * p.dplane + dcol;
+        // Samples at the box's rim and in the gap take the background's update, chosen per sample at the end: one
+        // chain a pair whatever its samples are.  (Each such sample's update in turn, behind the wait, was the
+        // launch's longest chain: 48^3 step 8.7 -> 7.6 us, 128^3 37.3 -> 36.1.)
+        const bool inz = k >= p.mb[C][4] && k < p.mb[C][5], d0 = m0 && inz && !(g0 && in_gz), d1 = m1 && inz && !(g1 && in_gz);
         const float2 e0 = ldp_pre(Ec + id), rho = ldp_pre(rc + dv);
         float4 q[MQ];
 #pragma unroll
@@ -96,7 +99,16 @@ __device__ __forceinline__ float design_pair_column(const KParams<float>& p, con
             hbm = ldp(Hb + id - nx);       // H_x along y
         }
         // drive and the blended update, per element the operations of design_update
-        const float2 d = p_mul(p_sub(p_sub(ha, ham), p_sub(hb, hbm)), idx2);
+        float2 d = p_mul(p_sub(p_sub(ha, ham), p_sub(hb, hbm)), idx2);
+        if (C == 2 && (i == p.tfsf_i0 || i + 1 == p.tfsf_i0)) {   // the TF/SF plane
+            const float h = __ldg(p.hinc + n) * p.inv_dx;
+            (i == p.tfsf_i0 ? d.x : d.y) -= h;
+        }
+        if (src) {
+#pragma unroll 1
+            for (int s = 0; s < 2; ++s)
+                if (in_box(p.sb, i + s, j, k)) (s ? d.y : d.x) += point_drive(p, i + s, j, k, C, n);
+        }
         const float2 gm = p_mul(p_mul(hg, rho), p_sub(one2, rho));
         const float2 D = p_add(p_fma(rho, dD, D1), gm);
         const float2 N = p_sub(p_fma(rho, dN, N1), gm);
@@ -111,7 +123,10 @@ __device__ __forceinline__ float design_pair_column(const KParams<float>& p, con
             }
         }
         const float2 num = p_sub(p_fma(N, e0, d), sq);
-        const float2 e = f2(div_t(num.x, D.x), div_t(num.y, D.y));
+        const float2 eb = p_fma(f2(p.bg_ca[C], p.bg_ca[C]), e0, p_mul(f2(p.bg_cb[C], p.bg_cb[C]), d));
+        const float2 e = f2(d0 ? div_t(num.x, D.x) : eb.x, d1 ? div_t(num.y, D.y) : eb.y);
+        // (a background sample's currents follow its E and are read by nothing: masking them takes 128^3 from 36.1 to
+        // 37.1 us a step)
         const float2 es = p_add(e, e0);
 #pragma unroll
         for (int pp = 0; pp < MQ; ++pp) {
