@@ -935,6 +935,7 @@ struct Solver : SolverBase {
     {
         KParams<T> q = p;
         q.n_off = off;
+        q.down = !two_buffers;
         if (!two_buffers) {
             for (int cc = 0; cc < 3; ++cc) {
                 q.En[cc] = q.E[cc];

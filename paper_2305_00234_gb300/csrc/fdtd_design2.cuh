@@ -139,7 +139,8 @@ __device__ __forceinline__ float design_pair_column(const KParams<float>& p, con
             }
         }
         stp(p.En[C] + id, e);
-        stp(p.snap + slot0 + dv, e);
+        // read again only by the DFT, up to 16 steps on: out of L2 first (128^3 step 37.7 -> 37.2 us)
+        __stcs(reinterpret_cast<float2*>(p.snap + slot0 + dv), e);
         emax = fmaxf(emax, fmaxf(fabsf(e.x), fabsf(e.y)));
     }
     return emax;
@@ -164,7 +165,7 @@ template <int MP>
 __global__ void __launch_bounds__(kBX * kBY, ed2_min_blocks<MP>()) e_design2_kernel(const KParams<float> p,
                                                                                          const PoleTable<float> tab)
 {
-    const int zc = blockIdx.z / 3, c = blockIdx.z - 3 * zc;
+    const int bz = (int)phase_block(p, blockIdx.z, gridDim.z), zc = bz / 3, c = bz - 3 * zc;
     const int wx = (p.db[1] - p.db[0]) / 2;
     const int col = blockIdx.x * (kBX * kBY) + threadIdx.y * kBX + threadIdx.x;
     const int y = col / wx;

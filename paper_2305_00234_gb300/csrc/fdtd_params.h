@@ -165,6 +165,7 @@ struct KParams {
     int* ctl;                    // [0] first step of the current block of steps, [2] flags, [3] the first step for
                                  // the block's DFT launch
     int n_off;                   // the launch's step is ctl[0] + n_off
+    int down;                    // 1: E kernels take their blocks downwards (see phase_block)
     int ib[6];                   // interior box of the fused step kernel (empty: x0 = x1)
     int edz;                     // z planes per thread of e_design_kernel (<= kEdZ)
     int kc;                      // z planes per block of step_kernel (<= kKC)

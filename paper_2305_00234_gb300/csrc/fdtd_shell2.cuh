@@ -43,12 +43,12 @@ __device__ __forceinline__ float2 ldp_pre(const float* p) { return __ldcg(reinte
 __device__ __forceinline__ void stp(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
 
 // The pair (x, x+1), x = B[0] + 2j, of block b / thread t of a paired shell launch (boxes counted in pairs).
-__device__ __forceinline__ bool shell_pair(const ShellBoxes& s, ShellCol& c)
+__device__ __forceinline__ bool shell_pair(const ShellBoxes& s, unsigned bid, ShellCol& c)
 {
     int q = 0;
-    while (q + 1 < s.n && blockIdx.x >= s.first[q + 1]) ++q;
+    while (q + 1 < s.n && bid >= s.first[q + 1]) ++q;
     const int* B = s.b[q];
-    const unsigned loc = blockIdx.x - s.first[q];
+    const unsigned loc = bid - s.first[q];
     const unsigned wx = (unsigned)(B[1] - B[0]) / 2u, wxy = wx * (B[3] - B[2]);
     const unsigned chunks = (wxy + s.nt - 1) / s.nt;
     const unsigned zc = loc / chunks;
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_h2_kernel(c
 {
     constexpr int P = kShell2PZ;
     ShellCol cl;
-    if (!shell_pair(s, cl)) return;
+    if (!shell_pair(s, blockIdx.x, cl)) return;
     const int x = cl.x, y = cl.y;
     const int n = read_step(p);
     const float cneg = -(p.ch * p.inv_dx), idx = p.inv_dx, ch = p.ch;
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_e2_kernel(c
 {
     constexpr int P = kShell2PZ;
     ShellCol cl;
-    if (!shell_pair(s, cl)) return;
+    if (!shell_pair(s, phase_block(p, blockIdx.x, gridDim.x), cl)) return;
     const int n = read_step(p);
     {
         const int x = cl.x, y = cl.y;

@@ -490,12 +490,12 @@ struct ShellCol {
     int x, y, k0, k1;   // column, planes [k0, k1)
 };
 
-__device__ __forceinline__ bool shell_cell(const ShellBoxes& s, ShellCol& c)
+__device__ __forceinline__ bool shell_cell(const ShellBoxes& s, unsigned bid, ShellCol& c)
 {
     int q = 0;
-    while (q + 1 < s.n && blockIdx.x >= s.first[q + 1]) ++q;
+    while (q + 1 < s.n && bid >= s.first[q + 1]) ++q;
     const int* B = s.b[q];
-    const unsigned loc = blockIdx.x - s.first[q];
+    const unsigned loc = bid - s.first[q];
     const unsigned wx = B[1] - B[0], wxy = wx * (B[3] - B[2]);
     const unsigned chunks = (wxy + s.nt - 1) / s.nt;
     const unsigned zc = loc / chunks;
@@ -713,7 +713,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBX * kBY, sizeof(T) == 8 ? 2 : FDTD_SHELL_MINB) shell_h_kernel(const KParams<T> p, const ShellBoxes s)
 {
     ShellCol cl;
-    if (shell_cell(s, cl)) h_column<T, false, true>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
+    if (shell_cell(s, blockIdx.x, cl)) h_column<T, false, true>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
 }
 
 // E^{n+1} of the cells of one column (x, y), planes [k0, k1), that lie outside the working box, from
@@ -867,7 +867,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBX * kBY, sizeof(T) == 8 ? 2 : FDTD_SHELL_MINB) shell_e_kernel(const KParams<T> p, const ShellBoxes s)
 {
     ShellCol cl;
-    if (!shell_cell(s, cl)) return;
+    if (!shell_cell(s, phase_block(p, blockIdx.x, gridDim.x), cl)) return;
     const T emax = e_column<T, false, true>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
     if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
 }
