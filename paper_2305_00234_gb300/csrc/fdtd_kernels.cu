@@ -153,7 +153,7 @@ cudaError_t graph_step(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& p
 template <typename T>
 cudaError_t graph_shell(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& p, const ShellBoxes& s, bool e_part)
 {
-    const dim3 grid(s.first[s.n]), b(kBX, s.nt / kBX);
+    const dim3 grid(s.first[s.n]), b(kBX, kShellBY);
     if constexpr (sizeof(T) == 4) {
         if (s.pair)
             return e_part ? graph_kernel(g, node, shell_e2_kernel, grid, b, 0, p, s)
@@ -230,48 +230,44 @@ cudaError_t launch_step(const KParams<T>& p, const StepMaps& m, cudaStream_t s, 
     return launch_chain(step_kernel<T>, g, dim3(kPX, kTY), StepSmem<T>::total, s, pdl, p, m);
 }
 
-// Shape of the shell launches: z planes per thread and threads per block, by an estimate of the busiest SM's time.
-// A column is a serial chain: with c blocks resident a plane (FP64: its arithmetic's latency) waits L and a plane
-// takes c t of the SM; an SM runs its b blocks C at a time, and every block costs the launch g.  L, t, g (us, t for
-// 256 threads) and C are read off steps of 48^3 to 192^3 grids and of 96 x 170 x 170 with every depth from 1 to 16.
-// What it decides: one full round of long columns instead of one and a little (96 x 170 x 170: depth 9, 608 blocks,
-// a step 60 us; depth 8, 704 blocks, 68; 128^3: depths 7 to 9 42 us, 6 47), and short columns, in blocks that spread
-// evenly, where a grid has few of them (48^3: depth 1 in blocks of 128 9.4 us, 4 in blocks of 256 12.9).  Past three
-// rounds only L/C + t a plane matters, which the depth does not change, and it stays at kLongColumn.
+// Shape of the shell launches: z planes per thread, by an estimate of the busiest SM's time.  A column is a serial
+// chain: with c blocks resident a plane (FP64: its arithmetic's latency) waits L and a plane takes c t of the SM; an SM
+// runs its b blocks C at a time, and every block costs the launch g.  L, t, g (us) and C are read off steps of
+// 48^3 to 192^3 grids and of 96 x 170 x 170 with every depth from 1 to 16.  What it decides: one full round of long
+// columns instead of one and a little (96 x 170 x 170: depth 9, 1216 blocks, a step 55.6 us; depth 8, 68 before), and
+// short columns where a grid has few of them (48^3: depth 1 7.3 us, 2 8.2, 4 11.2).  Past three rounds only L/C + t a
+// plane matters, which the depth does not change, and it stays at kLongColumn.
+// Blocks of 128 threads, not 256: they spread more evenly over the SMs (FP64 32^3 step 12.2 -> 10.8 us,
+// 88^3 19.8 -> 15.5, 121 x 81 x 95 23.9 -> 23.2, 75 x 61 x 83 11.9 -> 11.5, 128^3 and up within 1%).
 void shell_shape(ShellBoxes& s, int type_bytes)
 {
     const bool f64 = type_bytes == 8;
-    const double L = f64 ? 1.2 : 0.7, t256 = f64 ? 3.3 : (s.pair ? 0.45 : 0.25), g = 0.003;
-    const int resident256 = f64 ? 2 : 4, sms = 152;
-    auto blocks = [&](int kz, int nt) {
-        unsigned t = 0;
+    const double L = f64 ? 1.2 : 0.7, t = f64 ? 1.65 : (s.pair ? 0.225 : 0.125), g = 0.001;
+    const unsigned C = f64 ? 4 : 8, sms = 152;
+    auto blocks = [&](int kz) {
+        unsigned n = 0;
         for (int q = 0; q < s.n; ++q) {
             const int* B = s.b[q];
             const unsigned wxy = (unsigned)(B[1] - B[0]) / (s.pair ? 2u : 1u) * (unsigned)(B[3] - B[2]);
-            s.first[q] = t;
-            t += (wxy + nt - 1) / nt * (unsigned)((B[5] - B[4] + kz - 1) / kz);
+            s.first[q] = n;
+            n += (wxy + kShellNT - 1) / kShellNT * (unsigned)((B[5] - B[4] + kz - 1) / kz);
         }
-        s.first[s.n] = t;
-        return t;
+        s.first[s.n] = n;
+        return n;
     };
     constexpr int kLongColumn = 8;
     double best = 0.0;
     s.kz = 0;
-    for (int nt : {128, 256})
-        for (int kz = 1; kz <= kShellKZ; ++kz) {
-            const unsigned nb = blocks(kz, nt), b = (nb + sms - 1) / sms;
-            const unsigned C = resident256 * 256 / nt;
-            if (kz > kLongColumn && b > 3 * C) continue;
-            // FP32 blocks of 128 threads find fewer of their neighbours' rows in L1
-            const double t = t256 * nt / 256.0 * (nt < 256 && !f64 ? 1.05 : 1.0), wait = kz * L;
-            const double cost = (b / C) * (wait + kz * C * t) + (b % C ? wait + kz * (b % C) * t : 0.0) + g * nb;
-            if (s.kz == 0 || cost < best) {
-                best = cost;
-                s.kz = kz;
-                s.nt = nt;
-            }
+    for (int kz = 1; kz <= kShellKZ; ++kz) {
+        const unsigned nb = blocks(kz), b = (nb + sms - 1) / sms;
+        if (kz > kLongColumn && b > 3 * C) continue;
+        const double cost = (b / C) * (kz * L + kz * C * t) + (b % C ? kz * L + kz * (b % C) * t : 0.0) + g * nb;
+        if (s.kz == 0 || cost < best) {
+            best = cost;
+            s.kz = kz;
         }
-    blocks(s.kz, s.nt);
+    }
+    blocks(s.kz);
 }
 
 template <typename T>
@@ -279,7 +275,7 @@ cudaError_t launch_shell(const KParams<T>& p, const ShellBoxes& s, bool e_part, 
 {
     const unsigned nb = s.first[s.n];
     if (nb == 0) return cudaSuccess;
-    const dim3 b(kBX, s.nt / kBX);
+    const dim3 b(kBX, kShellBY);
     if constexpr (sizeof(T) == 4) {
         if (s.pair)
             return e_part ? launch_chain(shell_e2_kernel, dim3(nb), b, 0, st, pdl, p, s)

@@ -12,10 +12,12 @@ constexpr int kMaxFreq = 8;
 constexpr int kMaxBasis = 2 * kMaxFreq;
 constexpr int kBX = 32;
 constexpr int kBY = 8;
+constexpr int kShellBY = 4;       // shell blocks: kBX x kShellBY threads
+constexpr int kShellNT = kBX * kShellBY;
 constexpr int kReduceThreads = 256;
 constexpr int kMaxSnap = 16;      // steps per blocked DFT update (snapshot ring length)
 #ifndef FDTD_SHELL_MINB
-#define FDTD_SHELL_MINB 4
+#define FDTD_SHELL_MINB 8
 #endif
 #ifndef FDTD_KC
 #define FDTD_KC 8
@@ -92,7 +94,6 @@ struct ShellBoxes {
     int b[6][6];          // half-open x0, x1, y0, y1, z0, z1
     unsigned first[7];
     int kz;               // z planes per thread (<= kShellKZ)
-    int nt;               // threads per block (a multiple of kBX)
     int pair;             // 1: the paired kernels (a thread per two x-adjacent columns; every x bound even)
 };
 

@@ -17,7 +17,7 @@
 #define FDTD_SHELL2_PZ 1
 #endif
 #ifndef FDTD_SHELL2_MINB
-#define FDTD_SHELL2_MINB 4
+#define FDTD_SHELL2_MINB 8
 #endif
 
 namespace fdtd {
@@ -50,9 +50,9 @@ __device__ __forceinline__ bool shell_pair(const ShellBoxes& s, unsigned bid, Sh
     const int* B = s.b[q];
     const unsigned loc = bid - s.first[q];
     const unsigned wx = (unsigned)(B[1] - B[0]) / 2u, wxy = wx * (B[3] - B[2]);
-    const unsigned chunks = (wxy + s.nt - 1) / s.nt;
+    const unsigned chunks = (wxy + kShellNT - 1) / kShellNT;
     const unsigned zc = loc / chunks;
-    const unsigned t = (loc - zc * chunks) * s.nt + threadIdx.y * kBX + threadIdx.x;
+    const unsigned t = (loc - zc * chunks) * kShellNT + threadIdx.y * kBX + threadIdx.x;
     const unsigned yy = t / wx;
     c.x = B[0] + 2 * (int)(t - yy * wx);
     c.y = B[2] + (int)yy;
@@ -114,7 +114,7 @@ __device__ __forceinline__ void psi_store_p(float* const (&ps)[3][2], const PsiC
 }
 
 // H of the shell, one pair of columns per thread, planes [k0, k1) in batches of kShell2PZ.
-__global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_h2_kernel(const KParams<float> p, const ShellBoxes s)
+__global__ void __launch_bounds__(kShellNT, FDTD_SHELL2_MINB) shell_h2_kernel(const KParams<float> p, const ShellBoxes s)
 {
     constexpr int P = kShell2PZ;
     ShellCol cl;
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_h2_kernel(c
 
 // E of the shell cells outside the working box, one pair of columns per thread.  It may run concurrently
 // with the design-E kernel.
-__global__ void __launch_bounds__(kBX * kBY, FDTD_SHELL2_MINB) shell_e2_kernel(const KParams<float> p, const ShellBoxes s)
+__global__ void __launch_bounds__(kShellNT, FDTD_SHELL2_MINB) shell_e2_kernel(const KParams<float> p, const ShellBoxes s)
 {
     constexpr int P = kShell2PZ;
     ShellCol cl;

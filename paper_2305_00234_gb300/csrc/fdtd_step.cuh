@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(kPX * kTY, StepCfg<T>::MINB)
 }
 
 // ---- shell: per-cell kernels ----------------------------------------------------------------------
-// Block b -> box q; a block covers s.nt consecutive (x, y) columns of the box (x fastest, so a
+// Block b -> box q; a block covers kShellNT consecutive (x, y) columns of the box (x fastest, so a
 // warp reads and writes consecutive addresses even in boxes narrower than a warp), and each thread
 // marches s.kz (at most kShellKZ) planes of its column in batches of kShellPZ<T> planes whose loads are all
 // issued before any store.  The per-column set-up (box search, column coordinates, slab indices) is
@@ -497,9 +497,9 @@ __device__ __forceinline__ bool shell_cell(const ShellBoxes& s, unsigned bid, Sh
     const int* B = s.b[q];
     const unsigned loc = bid - s.first[q];
     const unsigned wx = B[1] - B[0], wxy = wx * (B[3] - B[2]);
-    const unsigned chunks = (wxy + s.nt - 1) / s.nt;
+    const unsigned chunks = (wxy + kShellNT - 1) / kShellNT;
     const unsigned zc = loc / chunks;
-    const unsigned t = (loc - zc * chunks) * s.nt + threadIdx.y * kBX + threadIdx.x;
+    const unsigned t = (loc - zc * chunks) * kShellNT + threadIdx.y * kBX + threadIdx.x;
     const unsigned yy = t / wx;
     c.x = B[0] + (int)(t - yy * wx);
     c.y = B[2] + (int)yy;
@@ -710,7 +710,7 @@ __device__ __forceinline__ void h_column(const KParams<T>& p, int x, int y, int 
 
 // H of the shell: one thread per column of a shell box (see shell_cell).
 template <typename T>
-__global__ void __launch_bounds__(kBX * kBY, sizeof(T) == 8 ? 2 : FDTD_SHELL_MINB) shell_h_kernel(const KParams<T> p, const ShellBoxes s)
+__global__ void __launch_bounds__(kShellNT, sizeof(T) == 8 ? 4 : FDTD_SHELL_MINB) shell_h_kernel(const KParams<T> p, const ShellBoxes s)
 {
     ShellCol cl;
     if (shell_cell(s, blockIdx.x, cl)) h_column<T, false, true>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
@@ -864,7 +864,7 @@ __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0,
 
 // E of the shell cells outside the design box.  It may run concurrently with the design-E kernel.
 template <typename T>
-__global__ void __launch_bounds__(kBX * kBY, sizeof(T) == 8 ? 2 : FDTD_SHELL_MINB) shell_e_kernel(const KParams<T> p, const ShellBoxes s)
+__global__ void __launch_bounds__(kShellNT, sizeof(T) == 8 ? 4 : FDTD_SHELL_MINB) shell_e_kernel(const KParams<T> p, const ShellBoxes s)
 {
     ShellCol cl;
     if (!shell_cell(s, phase_block(p, blockIdx.x, gridDim.x), cl)) return;
