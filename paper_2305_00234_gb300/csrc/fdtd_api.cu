@@ -407,6 +407,7 @@ struct Solver : SolverBase {
     bool fused = false;             // an interior box for the fused TMA step kernel exists
     int layout = 0;                 // fdtd_set_step_layout: 0 by size, 1 shell kernels only, 2 interior kernel
     bool use_pdl = true;            // step graphs with programmatic edges between phases (else captured)
+    bool one_e = false;             // their E phase is one launch
     bool pdl_built = false;         // a step graph with programmatic edges has been instantiated
     StepMaps maps[2]{};             // tensor maps of the buffers read by even / odd steps
     fdtd::ShellBoxes shell_around{};   // the cells around the interior box
@@ -1118,13 +1119,17 @@ struct Solver : SolverBase {
         auto direct = [&](int to) {
             const int s0 = s;
             for (; s < to; ++s) CK(launch_one_step(par(p, s, s - s0), s, false, mp));
-            if (s > s0) CK(fdtd::launch_block_end(p.ctl, s - s0, c->work));
+            if (s == s0) return;
+            CK(fdtd::launch_block_end(p.ctl, s - s0, c->work));
+            c->tim.launches++;
         };
         if ((s & 1) && s < n_to) direct(s + 1);
         if (use_pdl && !gx && n_to - s >= kGraphSteps) gx = build_pdl_graph(p, mp, kGraphSteps, nullptr);
-        for (; gx && n_to - s >= kGraphSteps; s += kGraphSteps) CK(cudaGraphLaunch(gx, c->work));
+        long long graphs = 0;
+        for (; gx && n_to - s >= kGraphSteps; s += kGraphSteps, ++graphs) CK(cudaGraphLaunch(gx, c->work));
         direct(n_to);
-        c->tim.launches += (long long)(n_to - n_from) * (interior() ? 4 : 3);
+        c->tim.launches += (long long)(n_to - n_from) * (interior() ? 4 : 3) + graphs;
+        if (one_e) c->tim.launches -= graphs * kGraphSteps;
     }
 
     void pm_check(const int* ctl_dev, int expect)
@@ -1356,6 +1361,11 @@ struct Solver : SolverBase {
             });
             phase([&] {
                 cudaGraphNode_t n = nullptr;
+                one_e = e == cudaSuccess && c->nd && !interior() && fdtd::graph_e_phase<T>(g, &n, q, shell(), htab, bucket, &e);
+                if (one_e) {
+                    if (e == cudaSuccess) cur.push_back(n);
+                    return;
+                }
                 if (e == cudaSuccess && has_shell && (e = fdtd::graph_shell<T>(g, &n, q, shell(), true)) == cudaSuccess)
                     cur.push_back(n);
                 if (e == cudaSuccess && c->nd && (e = fdtd::graph_e_design<T>(g, &n, q, htab, bucket)) == cudaSuccess)
@@ -1497,7 +1507,9 @@ struct Solver : SolverBase {
             c->tim.dft_launches += timed_blocks;
             c->tim.launches += nblk;
         }
-        c->tim.launches += ((interior() ? 3LL : 2LL) + (c->nd ? 1LL : 0LL)) * M;  // every kernel this run launched
+        // every kernel this run launched: a step's, and the two that begin and end a block
+        c->tim.launches += ((interior() ? 3LL : 2LL) + (c->nd ? 1LL : 0LL)) * M + 2 * nblk;
+        if (one_e) c->tim.launches -= M - timed_steps;
         c->tim.fused_step = fused ? 1 : 0;
         int hctl[4];
         CK(cudaMemcpyAsync(hctl, ctl, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->work));

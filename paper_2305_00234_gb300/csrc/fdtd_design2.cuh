@@ -161,13 +161,14 @@ constexpr int ed2_min_blocks()
 // One block: 256 column pairs in row order of component blockIdx.z % 3, p.edz planes each.  Every lane is
 // busy whatever the box's width (tiles of 32 x 8 pairs before: 96 x 84 x 108 voxels 38.8 -> 36.0 us a
 // launch, 32^3 voxels 9.4 -> 8.5 us).
+// block (bx, bz) of a launch with nz blocks in z, of nt threads
 template <int MP>
-__global__ void __launch_bounds__(kBX * kBY, ed2_min_blocks<MP>()) e_design2_kernel(const KParams<float> p,
-                                                                                         const PoleTable<float> tab)
+__device__ __forceinline__ void e_design2_block(const KParams<float>& p, const PoleTable<float>& tab, unsigned bx, unsigned bz,
+                                                unsigned nz, int nt)
 {
-    const int bz = (int)phase_block(p, blockIdx.z, gridDim.z), zc = bz / 3, c = bz - 3 * zc;
+    const int b = (int)phase_block(p, bz, nz), zc = b / 3, c = b - 3 * zc;
     const int wx = (p.db[1] - p.db[0]) / 2;
-    const int col = blockIdx.x * (kBX * kBY) + threadIdx.y * kBX + threadIdx.x;
+    const int col = (int)bx * nt + threadIdx.y * kBX + threadIdx.x;
     const int y = col / wx;
     const int i = p.db[0] + 2 * (col - y * wx);
     const int j = p.db[2] + y;
@@ -178,6 +179,33 @@ __global__ void __launch_bounds__(kBX * kBY, ed2_min_blocks<MP>()) e_design2_ker
                      : c == 1 ? design_pair_column<MP, 1>(p, tab, i, j, k0, k1, n)
                               : design_pair_column<MP, 2>(p, tab, i, j, k0, k1, n);
     if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
+}
+
+template <int MP>
+__global__ void __launch_bounds__(kBX * kBY, ed2_min_blocks<MP>()) e_design2_kernel(const KParams<float> p,
+                                                                                         const PoleTable<float> tab)
+{
+    e_design2_block<MP>(p, tab, blockIdx.x, blockIdx.z, gridDim.z, kBX * kBY);
+}
+
+// The whole E phase in one launch (SP, DP: paired shell and design kernels): the design box's blocks, gx column
+// groups by gz z chunks and components, then the shell's.
+template <bool SP, bool DP, int MP>
+__global__ void __launch_bounds__(kShellNT, 8) e_phase_kernel(const KParams<float> p, const ShellBoxes s, const PoleTable<float> tab,
+                                                              unsigned gx, unsigned gz)
+{
+    const unsigned nd = gx * gz;
+    if (blockIdx.x < nd) {
+        const unsigned bz = blockIdx.x / gx, bx = blockIdx.x - bz * gx;
+        if constexpr (DP)
+            e_design2_block<MP>(p, tab, bx, bz, gz, kShellNT);
+        else
+            e_design_block<float, MP>(p, tab, bx, bz, gz, kShellNT);
+    } else if constexpr (SP) {
+        shell_e2_block(p, s, blockIdx.x - nd);
+    } else {
+        shell_e_block(p, s, blockIdx.x - nd);
+    }
 }
 
 }  // namespace fdtd

@@ -166,11 +166,11 @@ cudaError_t graph_shell(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& 
 // Grid of the design-E kernel: one block per (p.edz planes, component) of 256 columns (column pairs for
 // the paired kernel) in row order.
 template <typename T>
-static dim3 design_grid(const KParams<T>& p)
+static dim3 design_grid(const KParams<T>& p, int nt = kBX * kBY)
 {
     const unsigned nxy = (unsigned)((p.db[1] - p.db[0]) / (p.ed_pair ? 2 : 1)) * (unsigned)(p.db[3] - p.db[2]);
     const unsigned nz = (unsigned)(p.db[5] - p.db[4]);
-    return dim3((nxy + kBX * kBY - 1) / (kBX * kBY), 1, 3 * ((nz + p.edz - 1) / p.edz));
+    return dim3((nxy + nt - 1) / nt, 1, 3 * ((nz + p.edz - 1) / p.edz));
 }
 
 template <typename T>
@@ -191,6 +191,31 @@ cudaError_t graph_e_design(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T
     case 8: return graph_kernel(g, node, e_design_kernel<T, 8>, grid, b, 0, p, tab);
     default: return graph_kernel(g, node, e_design_kernel<T, 16>, grid, b, 0, p, tab);
     }
+}
+
+// The E phase as one launch (FP32, up to 4 poles a component), where the launches are what the phase costs: columns
+// of one plane and, with the one-sample design kernel, blocks that are resident at once; false: it takes two.
+// 48^3 step 7.6 -> 7.25 us, 56^3 8.35 -> 8.05, 64^3 10.4 -> 9.8, 96 x 64 x 48 10.65 -> 10.2, 44^3 (one-sample) 7.0 -> 6.5.
+// With longer columns the design box's blocks only hold the shell's up (72^3 11.2 -> 12.0), and so do the one-sample
+// kernel's past one round (56^3 8.45 -> 8.85).
+template <typename T>
+bool graph_e_phase(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& p, const ShellBoxes& s, const PoleTable<T>& tab,
+                   int bucket, cudaError_t* e)
+{
+    if constexpr (sizeof(T) == 4) {
+        const dim3 dg = design_grid(p, kShellNT), grid(dg.x * dg.z + s.first[s.n]), b(kBX, kShellBY);
+        if (bucket > 4 || s.kz > 1 || (!p.ed_pair && grid.x > 8 * 152)) return false;
+        void (*k)(KParams<float>, ShellBoxes, PoleTable<float>, unsigned, unsigned);
+        if (bucket == 0)
+            k = p.ed_pair ? (s.pair ? e_phase_kernel<true, true, 0> : e_phase_kernel<false, true, 0>)
+                          : (s.pair ? e_phase_kernel<true, false, 0> : e_phase_kernel<false, false, 0>);
+        else
+            k = p.ed_pair ? (s.pair ? e_phase_kernel<true, true, 4> : e_phase_kernel<false, true, 4>)
+                          : (s.pair ? e_phase_kernel<true, false, 4> : e_phase_kernel<false, false, 4>);
+        *e = graph_kernel(g, node, k, grid, b, 0, p, s, tab, dg.x, dg.z);
+        return true;
+    }
+    return false;
 }
 
 template <typename T>
@@ -449,6 +474,8 @@ cudaError_t launch_rho_scatter(const void* src, int dtype, long long n, const lo
     template cudaError_t graph_step<T>(cudaGraph_t, cudaGraphNode_t*, const KParams<T>&, const StepMaps&); \
     template cudaError_t graph_shell<T>(cudaGraph_t, cudaGraphNode_t*, const KParams<T>&, const ShellBoxes&, bool); \
     template cudaError_t graph_e_design<T>(cudaGraph_t, cudaGraphNode_t*, const KParams<T>&, const PoleTable<T>&, int); \
+    template bool graph_e_phase<T>(cudaGraph_t, cudaGraphNode_t*, const KParams<T>&, const ShellBoxes&, const PoleTable<T>&, int, \
+                                   cudaError_t*);                                                        \
     template cudaError_t graph_dft<T>(cudaGraph_t, cudaGraphNode_t*, const DParams<T>&, int);           \
     template cudaError_t launch_step<T>(const KParams<T>&, const StepMaps&, cudaStream_t, bool);         \
     template cudaError_t launch_shell<T>(const KParams<T>&, const ShellBoxes&, bool, cudaStream_t, bool); \

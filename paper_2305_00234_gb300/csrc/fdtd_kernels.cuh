@@ -360,12 +360,14 @@ __device__ __forceinline__ unsigned phase_block(const KParams<T>& p, unsigned b,
     return p.down ? n - 1 - b : b;
 }
 
+// block (bx, bz) of a launch with nz blocks in z, of nt threads
 template <typename T, int MP>
-__global__ void __launch_bounds__(kBX * kBY, ed_min_blocks<T, MP>()) e_design_kernel(const KParams<T> p, const PoleTable<T> tab)
+__device__ __forceinline__ void e_design_block(const KParams<T>& p, const PoleTable<T>& tab, unsigned bx, unsigned bz, unsigned nz,
+                                               int nt)
 {
-    const int bz = (int)phase_block(p, blockIdx.z, gridDim.z), zc = bz / 3, c = bz - 3 * zc;
+    const int b = (int)phase_block(p, bz, nz), zc = b / 3, c = b - 3 * zc;
     const int dnx = p.db[1] - p.db[0];   // columns in row order, kBX * kBY per block
-    const int col = blockIdx.x * (kBX * kBY) + threadIdx.y * kBX + threadIdx.x;
+    const int col = (int)bx * nt + threadIdx.y * kBX + threadIdx.x;
     const int y = col / dnx;
     const int i = p.db[0] + (col - y * dnx), j = p.db[2] + y;
     const int k0 = p.db[4] + zc * p.edz, k1 = min(p.db[5], k0 + p.edz);
@@ -375,6 +377,12 @@ __global__ void __launch_bounds__(kBX * kBY, ed_min_blocks<T, MP>()) e_design_ke
                  : c == 1 ? e_design_column<T, MP, 1, false, true>(p, tab, i, j, k0, k1, n)
                           : e_design_column<T, MP, 2, false, true>(p, tab, i, j, k0, k1, n);
     if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
+}
+
+template <typename T, int MP>
+__global__ void __launch_bounds__(kBX * kBY, ed_min_blocks<T, MP>()) e_design_kernel(const KParams<T> p, const PoleTable<T> tab)
+{
+    e_design_block<T, MP>(p, tab, blockIdx.x, blockIdx.z, gridDim.z, kBX * kBY);
 }
 
 // ---------------------------------------------------------------------------------------------

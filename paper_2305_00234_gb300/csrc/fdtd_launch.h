@@ -18,6 +18,10 @@ template <typename T>
 cudaError_t graph_shell(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& p, const ShellBoxes& s, bool e_part);
 template <typename T>
 cudaError_t graph_e_design(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& p, const PoleTable<T>& tab, int bucket);
+// the whole E phase as one node, where it can be (else false)
+template <typename T>
+bool graph_e_phase(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& p, const ShellBoxes& s, const PoleTable<T>& tab,
+                   int bucket, cudaError_t* e);
 template <typename T>
 cudaError_t graph_dft(cudaGraph_t g, cudaGraphNode_t* node, const DParams<T>& d, int cnt);
 // begin and end of a block of cnt steps: the first step for the DFT launch, the step counter moved on

@@ -239,11 +239,11 @@ __global__ void __launch_bounds__(kShellNT, FDTD_SHELL2_MINB) shell_h2_kernel(co
 
 // E of the shell cells outside the working box, one pair of columns per thread.  It may run concurrently
 // with the design-E kernel.
-__global__ void __launch_bounds__(kShellNT, FDTD_SHELL2_MINB) shell_e2_kernel(const KParams<float> p, const ShellBoxes s)
+__device__ __forceinline__ void shell_e2_block(const KParams<float>& p, const ShellBoxes& s, unsigned bid)
 {
     constexpr int P = kShell2PZ;
     ShellCol cl;
-    if (!shell_pair(s, phase_block(p, blockIdx.x, gridDim.x), cl)) return;
+    if (!shell_pair(s, phase_block(p, bid, s.first[s.n]), cl)) return;
     const int n = read_step(p);
     {
         const int x = cl.x, y = cl.y;
@@ -393,6 +393,11 @@ __global__ void __launch_bounds__(kShellNT, FDTD_SHELL2_MINB) shell_e2_kernel(co
         }
         if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
     }
+}
+
+__global__ void __launch_bounds__(kShellNT, FDTD_SHELL2_MINB) shell_e2_kernel(const KParams<float> p, const ShellBoxes s)
+{
+    shell_e2_block(p, s, blockIdx.x);
 }
 
 }  // namespace fdtd

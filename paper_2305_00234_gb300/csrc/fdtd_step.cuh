@@ -864,12 +864,18 @@ __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0,
 
 // E of the shell cells outside the design box.  It may run concurrently with the design-E kernel.
 template <typename T>
-__global__ void __launch_bounds__(kShellNT, sizeof(T) == 8 ? 4 : FDTD_SHELL_MINB) shell_e_kernel(const KParams<T> p, const ShellBoxes s)
+__device__ __forceinline__ void shell_e_block(const KParams<T>& p, const ShellBoxes& s, unsigned bid)
 {
     ShellCol cl;
-    if (!shell_cell(s, phase_block(p, blockIdx.x, gridDim.x), cl)) return;
+    if (!shell_cell(s, phase_block(p, bid, s.first[s.n]), cl)) return;
     const T emax = e_column<T, false, true>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
     if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kShellNT, sizeof(T) == 8 ? 4 : FDTD_SHELL_MINB) shell_e_kernel(const KParams<T> p, const ShellBoxes s)
+{
+    shell_e_block(p, s, blockIdx.x);
 }
 
 }  // namespace fdtd
