@@ -33,9 +33,9 @@ constexpr int kMaxSnap = 16;      // steps per blocked DFT update (snapshot ring
 #endif
 constexpr int kEdZ = FDTD_ED_Z;     // most z planes per thread in the design-E kernel
 constexpr int kEdPZ = FDTD_ED_PZ;   // of which loaded per batch
-// z planes per batch of loads in the one-cell shell kernels.  FP32: with 4 blocks of 256 threads an SM the other
+// z planes per batch of loads in the one-cell shell kernels.  FP32: with 1024 threads an SM the other
 // warps cover a plane's loads, and a second plane's only take registers (75 x 61 x 83 step 12.6 -> 11.9 us, 121 x 81 x
-// 95 25.1 -> 23.9); FP64 has 2 blocks, and 32^3 takes 12.5 us a step with one plane, 12.2 with two.
+// 95 25.1 -> 23.9); FP64 has 512, and 32^3 takes 12.5 us a step with one plane, 12.2 with two.
 template <typename T>
 constexpr int kShellPZ = sizeof(T) == 8 ? 2 : 1;
 constexpr int kShellKZ = FDTD_SHELL_KZ;   // most z planes per thread in the shell kernels (even)

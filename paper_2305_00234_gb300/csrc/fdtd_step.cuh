@@ -1,7 +1,8 @@
 // Background step for sm_103a: H^{n+1/2} everywhere and E^{n+1} for every cell outside the design
 // box (Yee update of Eqs. (Maxwells)a-c with the background material, CFS-CPML psi in the edge slabs,
-// the TF/SF correction and point sources), reading E^n / H^{n-1/2} from one buffer of each pair and
-// writing the other.  The grid is split in two:
+// the TF/SF correction and point sources).  Grids below the host's cell limits are one box of the shell
+// kernels below, updated in place; larger ones are split in two, reading E^n / H^{n-1/2} from one buffer of
+// each pair and writing the other:
 //
 // * an interior box of tiles (the last column or row may be partial), away from the walls and the CPML
 //   slabs, updated by step_kernel in one pass: 48 B per cell (each field word read once and written
