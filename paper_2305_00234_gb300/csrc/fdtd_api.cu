@@ -588,7 +588,9 @@ struct Solver : SolverBase {
         }
         p.edz = 1;
         p.ed_pair = design_pairable() ? 1 : 0;
-        if (c->nd) p.edz = fdtd::design_planes((p.ed_pair ? c->dn[0] / 2 : c->dn[0]) * c->dn[1], c->dn[2]);
+        if (c->nd)
+            p.edz = fdtd::design_planes((p.ed_pair ? c->dn[0] / 2 : c->dn[0]) * c->dn[1], c->dn[2], sizeof(T) == 8,
+                                        p.ed_pair && bucket <= 4 && shell_all.kz == 1 ? shell_all.first[shell_all.n] : 0);
         p.blowup = (T)1e30;
         p.n_steps = d.n_steps;
         p.tfsf_i0 = -1;

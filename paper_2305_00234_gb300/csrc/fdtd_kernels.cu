@@ -351,18 +351,28 @@ cudaError_t launch_block_end(int* ctl, int cnt, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// Columns of kEdZ planes, halved while the launch has fewer than FDTD_ED_MINCOLS blocks (default: one
-// wave of five resident blocks per SM; measured 3.7% faster than two blocks per SM on the 96 x 170 x 170
-// paper grid, whose design box is 26 cells deep in x).
-#ifndef FDTD_ED_MINCOLS
-#define FDTD_ED_MINCOLS (5 * 152)
-#endif
-int design_planes(int columns, int dnz)
+// Planes per thread of the design-E kernel.  FP32: short columns spread evenly and leave more loads in flight,
+// long ones prefetch their next plane, which counts the more the less of the box L2 holds.  Steps measured with 1, 2, 3,
+// 5, 8 planes, by the rounds (of 4 blocks an SM) that a launch of one-plane columns takes: 112^3 (2 rounds) 25.3 25.3
+// 25.7 27.6 30.2 us; 96 x 170 x 170 (3) 60.5 60.2 60.6 60.3 63.0; 128^3 (3) 36.7 36.2 36.3 37.5 39.9; 192^3 (9) 124.1
+// 120.5 120.6 121.3 123.3; 256^3 (20) 276.7 268.6 268.3 269.3 271.5; 512 x 512 x 384 (121) 1794 1691 1658 1644 1649.
+// other_blocks: the shell's blocks of kShellNT threads, where the E phase is one launch: two planes where that makes it
+// one round (64^3, 1024 of them: a step 8.1 -> 7.55 us).
+// FP64: columns of kEdZ planes, halved while the launch has fewer than five blocks an SM.
+int design_planes(int columns, int dnz, bool f64, unsigned other_blocks)
 {
-    const unsigned gxy = ((unsigned)columns + kBX * kBY - 1) / (kBX * kBY);
-    int edz = kEdZ;
-    while (edz > 1 && gxy * 3 * (((unsigned)dnz + edz - 1) / edz) < FDTD_ED_MINCOLS) edz = (edz + 1) / 2;
-    return edz;
+    constexpr unsigned sms = 152;
+    const unsigned gxy = ((unsigned)columns + kBX * kBY - 1) / (kBX * kBY), one = gxy * 3 * (unsigned)dnz;
+    if (f64) {
+        int edz = kEdZ;
+        while (edz > 1 && gxy * 3 * (((unsigned)dnz + edz - 1) / edz) < 5 * sms) edz = (edz + 1) / 2;
+        return edz;
+    }
+    if (other_blocks) {
+        const unsigned g = ((unsigned)columns + kShellNT - 1) / kShellNT;
+        if (other_blocks + 3 * g * dnz > 8 * sms && other_blocks + 3 * g * ((dnz + 1) / 2) <= 8 * sms) return 2;
+    }
+    return one < 2 * 4 * sms ? 1 : (one < 12 * 4 * sms ? 2 : (one < 40 * 4 * sms ? 3 : 5));
 }
 
 template <typename T>

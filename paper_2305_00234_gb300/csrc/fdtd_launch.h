@@ -38,7 +38,7 @@ cudaError_t launch_dft(const DParams<T>& d, int cnt, cudaStream_t s, bool pdl = 
 void shell_shape(ShellBoxes& s, int type_bytes);   // picks s.kz, fills s.first
 template <typename T>
 cudaError_t launch_shell(const KParams<T>& p, const ShellBoxes& s, bool e_part, cudaStream_t st, bool pdl = false);
-int design_planes(int columns, int dnz);   // z planes per thread of the design-E kernel
+int design_planes(int columns, int dnz, bool f64, unsigned other_blocks);   // z planes per thread of the design-E kernel
 template <typename T>
 cudaError_t launch_grad(const GParams<T>& g, unsigned nblocks, cudaStream_t s);
 cudaError_t launch_gap_gather(const double2* dft, long long nd, int nf, const int* db, int dnx, int dny, const int* gb,
