@@ -366,6 +366,17 @@ int halo(double R) { return (int)std::ceil(R) - 1; }
 // The scratch of a radius: the normalising sums' table, the blocks' shared data (16-byte aligned: 8 | table words).
 size_t table_bytes(int n) { return table_words(n) * sizeof(long long) + sizeof(ConeMeta); }
 
+// A kernel's limit of dynamic shared memory is the device's, whoever launches: every call sets it to the largest
+// radius's need, so that no call can lower it between another thread's setting and its launch.
+template <typename K>
+cudaError_t allow_smem(K kernel, size_t most)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
+size_t cone_smem_bytes(int n) { return ConeTile(n).meta + sizeof(ConeMeta); }
+size_t table_smem_bytes(int n) { return table_words(n) * sizeof(long long); }
+
 cudaError_t conv(const float* in, float* out, const long long* T, bool normalise, float* proj, int nx, int ny, int nz,
                  double R, double beta, double eta, const ConeRows& rows, cudaStream_t s)
 {
@@ -385,21 +396,19 @@ cudaError_t conv(const float* in, float* out, const long long* T, bool normalise
     a.eta = (float)eta;
     a.pden = (float)(std::tanh(beta * eta) + std::tanh(beta * (1.0 - eta)));
     const bool vec = nx % 4 == 0 && (uintptr_t)in % 16 == 0;
-    const size_t smem = ConeTile(rows.n).meta + sizeof(ConeMeta);
     const auto k = vec ? cone_kernel<true> : cone_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, cone_smem_bytes(kMaxHalo));
     if (e != cudaSuccess) return e;
     const dim3 g((unsigned)((nx + kOX - 1) / kOX) * (unsigned)nz, (ny + kTY - 1) / kTY);   // z in grid x: no limit of 65535
-    k<<<g, kThreads, smem, s>>>(a);
+    k<<<g, kThreads, cone_smem_bytes(rows.n), s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t build_table(long long* T, const ConeRows& rows, double R, cudaStream_t s)
 {
-    const size_t smem = table_words(rows.n) * sizeof(long long);
-    cudaError_t e = cudaFuncSetAttribute(table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(table_kernel, table_smem_bytes(kMaxHalo));
     if (e != cudaSuccess) return e;
-    table_kernel<<<1, 1024, smem, s>>>(T, rows, (float)R);
+    table_kernel<<<1, 1024, table_smem_bytes(rows.n), s>>>(T, rows, (float)R);
     return cudaGetLastError();
 }
 
