@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kShellNT, 8) e_phase_kernel(const KParams<floa
     } else if constexpr (SP) {
         shell_e2_block(p, s, blockIdx.x - nd);
     } else {
-        shell_e_block(p, s, blockIdx.x - nd);
+        shell_e_block<float, 1>(p, s, blockIdx.x - nd);   // columns of one plane
     }
 }
 

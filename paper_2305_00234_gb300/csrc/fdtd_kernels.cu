@@ -159,8 +159,13 @@ cudaError_t graph_shell(cudaGraph_t g, cudaGraphNode_t* node, const KParams<T>& 
             return e_part ? graph_kernel(g, node, shell_e2_kernel, grid, b, 0, p, s)
                           : graph_kernel(g, node, shell_h2_kernel, grid, b, 0, p, s);
     }
-    return e_part ? graph_kernel(g, node, shell_e_kernel<T>, grid, b, 0, p, s)
-                  : graph_kernel(g, node, shell_h_kernel<T>, grid, b, 0, p, s);
+    if constexpr (sizeof(T) == 4) {
+        if (s.pz == 1)
+            return e_part ? graph_kernel(g, node, shell_e_kernel<T, 1>, grid, b, 0, p, s)
+                          : graph_kernel(g, node, shell_h_kernel<T, 1>, grid, b, 0, p, s);
+    }
+    return e_part ? graph_kernel(g, node, shell_e_kernel<T, 2>, grid, b, 0, p, s)
+                  : graph_kernel(g, node, shell_h_kernel<T, 2>, grid, b, 0, p, s);
 }
 
 // Grid of the design-E kernel: one block per (p.edz planes, component) of 256 columns (column pairs for
@@ -264,9 +269,10 @@ cudaError_t launch_step(const KParams<T>& p, const StepMaps& m, cudaStream_t s, 
 // plane matters, which the depth does not change, and it stays at kLongColumn.
 // Blocks of 128 threads, not 256: they spread more evenly over the SMs (FP64 32^3 step 12.2 -> 10.8 us,
 // 88^3 19.8 -> 15.5, 121 x 81 x 95 23.9 -> 23.2, 75 x 61 x 83 11.9 -> 11.5, 128^3 and up within 1%).
-void shell_shape(ShellBoxes& s, int type_bytes)
+void shell_shape(ShellBoxes& s, int type_bytes, size_t ncell)
 {
     const bool f64 = type_bytes == 8;
+    s.pz = f64 || ncell >= kShellTwoPlaneCells ? 2 : 1;
     const double L = f64 ? 1.2 : 0.7, t = f64 ? 1.65 : (s.pair ? 0.225 : 0.125), g = 0.001;
     const unsigned C = f64 ? 4 : 8, sms = 152;
     auto blocks = [&](int kz) {
@@ -306,8 +312,13 @@ cudaError_t launch_shell(const KParams<T>& p, const ShellBoxes& s, bool e_part, 
             return e_part ? launch_chain(shell_e2_kernel, dim3(nb), b, 0, st, pdl, p, s)
                           : launch_chain(shell_h2_kernel, dim3(nb), b, 0, st, pdl, p, s);
     }
-    return e_part ? launch_chain(shell_e_kernel<T>, dim3(nb), b, 0, st, pdl, p, s)
-                  : launch_chain(shell_h_kernel<T>, dim3(nb), b, 0, st, pdl, p, s);
+    if constexpr (sizeof(T) == 4) {
+        if (s.pz == 1)
+            return e_part ? launch_chain(shell_e_kernel<T, 1>, dim3(nb), b, 0, st, pdl, p, s)
+                          : launch_chain(shell_h_kernel<T, 1>, dim3(nb), b, 0, st, pdl, p, s);
+    }
+    return e_part ? launch_chain(shell_e_kernel<T, 2>, dim3(nb), b, 0, st, pdl, p, s)
+                  : launch_chain(shell_h_kernel<T, 2>, dim3(nb), b, 0, st, pdl, p, s);
 }
 
 template <typename T>

@@ -33,11 +33,15 @@ constexpr int kMaxSnap = 16;      // steps per blocked DFT update (snapshot ring
 #endif
 constexpr int kEdZ = FDTD_ED_Z;     // most z planes per thread in the design-E kernel
 constexpr int kEdPZ = FDTD_ED_PZ;   // of which loaded per batch
-// z planes per batch of loads in the one-cell shell kernels.  FP32: with 1024 threads an SM the other
-// warps cover a plane's loads, and a second plane's only take registers (75 x 61 x 83 step 12.6 -> 11.9 us, 121 x 81 x
-// 95 25.1 -> 23.9); FP64 has 512, and 32^3 takes 12.5 us a step with one plane, 12.2 with two.
+// z planes per batch of loads in the one-cell shell kernels.  FP32: while a grid's state stays in L2, the other warps of
+// an SM's 1024 threads cover a plane's loads, and a second plane's only take registers; past it the loads wait on
+// DRAM, and two planes of them in flight pay.  A step with one / two planes a batch: 75 x 61 x 83 11.0 / 11.2 us, 121 x 81 x 95
+// 20.2 / 21.4, 131 x 130 x 132 39.6 / 42.6; 141 x 140 x 142 50.7 / 49.1, 161 x 160 x 162 79.9 / 73.0, 241 x 240 x 242 266 /
+// 218, 301 x 300 x 302 512 / 411; beside an interior kernel (256^3, odd x CPML) 249 / 233.  The line lies between the
+// third and the fourth pair.  FP64 has 512 threads an SM, and 32^3 takes 12.5 us a step with one plane, 12.2 with two.
 template <typename T>
 constexpr int kShellPZ = sizeof(T) == 8 ? 2 : 1;
+constexpr size_t kShellTwoPlaneCells = 2500000;   // FP32 grids of this many cells and up: two
 constexpr int kShellKZ = FDTD_SHELL_KZ;   // most z planes per thread in the shell kernels (even)
 constexpr int kKC = FDTD_KC;      // z planes per block of the fused step kernel
 
@@ -94,6 +98,7 @@ struct ShellBoxes {
     int b[6][6];          // half-open x0, x1, y0, y1, z0, z1
     unsigned first[7];
     int kz;               // z planes per thread (<= kShellKZ)
+    int pz;               // one-cell kernels: z planes per batch of loads, 1 or 2
     int pair;             // 1: the paired kernels (a thread per two x-adjacent columns; every x bound even)
 };
 

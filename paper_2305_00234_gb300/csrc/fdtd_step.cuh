@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kPX * kTY, StepCfg<T>::MINB)
 // ---- shell: per-cell kernels ----------------------------------------------------------------------
 // Block b -> box q; a block covers kShellNT consecutive (x, y) columns of the box (x fastest, so a
 // warp reads and writes consecutive addresses even in boxes narrower than a warp), and each thread
-// marches s.kz (at most kShellKZ) planes of its column in batches of kShellPZ<T> planes whose loads are all
+// marches s.kz (at most kShellKZ) planes of its column in batches of P (s.pz) planes whose loads are all
 // issued before any store.  The per-column set-up (box search, column coordinates, slab indices) is
 // paid once per s.kz planes; cell and psi offsets are 32-bit (a grid holds fewer than 2^31
 // cells) and advance by a fixed stride per plane.
@@ -593,10 +593,9 @@ __device__ __forceinline__ T stretch_v(T d, const T* __restrict__ tab, int s, T&
 // batch's own.  CG: state loads bypass L1 (for a persistent kernel whose earlier work items on the
 // same SM may hold stale lines).  PDL: the caller has not waited for the phase before; the first batch's
 // H and psi_H loads come first.
-template <typename T, bool CG, bool PDL = false>
+template <typename T, bool CG, bool PDL = false, int P = kShellPZ<T>>
 __device__ __forceinline__ void h_column(const KParams<T>& p, int x, int y, int k0, int k1, int n)
 {
-    constexpr int P = kShellPZ<T>;
     const T cneg = -(p.ch * p.inv_dx), idx = p.inv_dx, ch = p.ch;
     const T einc_n = p.tfsf_i0 >= 0 ? __ldg(p.einc + n) : T(0);
     const bool tf = x == p.tfsf_i0 - 1;   // H_y here is scattered field
@@ -710,11 +709,11 @@ __device__ __forceinline__ void h_column(const KParams<T>& p, int x, int y, int 
 }
 
 // H of the shell: one thread per column of a shell box (see shell_cell).
-template <typename T>
+template <typename T, int P>
 __global__ void __launch_bounds__(kShellNT, sizeof(T) == 8 ? 4 : FDTD_SHELL_MINB) shell_h_kernel(const KParams<T> p, const ShellBoxes s)
 {
     ShellCol cl;
-    if (shell_cell(s, blockIdx.x, cl)) h_column<T, false, true>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
+    if (shell_cell(s, blockIdx.x, cl)) h_column<T, false, true, P>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
 }
 
 // E^{n+1} of the cells of one column (x, y), planes [k0, k1), that lie outside the working box, from
@@ -722,10 +721,9 @@ __global__ void __launch_bounds__(kShellNT, sizeof(T) == 8 ? 4 : FDTD_SHELL_MINB
 // h_column, with H_x, H_y of the plane below a batch carried over.  Returns the largest |E| sum seen
 // on a checked step (0 otherwise).  PDL: the caller has not waited for the phase before; the first batch's
 // E and psi_E loads come first.
-template <typename T, bool CG, bool PDL = false>
+template <typename T, bool CG, bool PDL = false, int P = kShellPZ<T>>
 __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0, int k1, int n)
 {
-    constexpr int P = kShellPZ<T>;
     T emax = T(0);
     {
         const T hinc_n = p.tfsf_i0 >= 0 ? __ldg(p.hinc + n) : T(0);
@@ -864,19 +862,19 @@ __device__ __forceinline__ T e_column(const KParams<T>& p, int x, int y, int k0,
 }
 
 // E of the shell cells outside the design box.  It may run concurrently with the design-E kernel.
-template <typename T>
+template <typename T, int P>
 __device__ __forceinline__ void shell_e_block(const KParams<T>& p, const ShellBoxes& s, unsigned bid)
 {
     ShellCol cl;
     if (!shell_cell(s, phase_block(p, bid, s.first[s.n]), cl)) return;
-    const T emax = e_column<T, false, true>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
+    const T emax = e_column<T, false, true, P>(p, cl.x, cl.y, cl.k0, cl.k1, read_step(p));
     if (!(emax < p.blowup)) atomicOr(p.ctl + 2, 1);
 }
 
-template <typename T>
+template <typename T, int P>
 __global__ void __launch_bounds__(kShellNT, sizeof(T) == 8 ? 4 : FDTD_SHELL_MINB) shell_e_kernel(const KParams<T> p, const ShellBoxes s)
 {
-    shell_e_block(p, s, blockIdx.x);
+    shell_e_block<T, P>(p, s, blockIdx.x);
 }
 
 }  // namespace fdtd
