@@ -584,7 +584,7 @@ struct Solver : SolverBase {
         for (int m = 0; m < 2; ++m) dp[m].ctl = ctl;
         for (fdtd::ShellBoxes* b : {&shell_around, &shell_all}) {
             b->pair = shell_pairable(p, *b) ? 1 : 0;
-            fdtd::shell_shape(*b, (int)sizeof(T), c->ncell);
+            fdtd::shell_shape(*b, (int)sizeof(T), c->ncell, b == &shell_around);
         }
         p.edz = 1;
         p.ed_pair = design_pairable() ? 1 : 0;

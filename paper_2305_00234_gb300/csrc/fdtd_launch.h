@@ -35,7 +35,8 @@ template <typename T>
 cudaError_t launch_e_design(const KParams<T>& p, const PoleTable<T>& tab, int bucket, cudaStream_t s, bool pdl = false);
 template <typename T>
 cudaError_t launch_dft(const DParams<T>& d, int cnt, cudaStream_t s, bool pdl = false);
-void shell_shape(ShellBoxes& s, int type_bytes, size_t ncell);   // picks s.kz and s.pz, fills s.first
+// picks s.kz and s.pz, fills s.first; beside: launched next to the interior kernel
+void shell_shape(ShellBoxes& s, int type_bytes, size_t ncell, bool beside);
 template <typename T>
 cudaError_t launch_shell(const KParams<T>& p, const ShellBoxes& s, bool e_part, cudaStream_t st, bool pdl = false);
 int design_planes(int columns, int dnz, bool f64, unsigned other_blocks);   // z planes per thread of the design-E kernel
