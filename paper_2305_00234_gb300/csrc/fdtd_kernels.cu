@@ -267,10 +267,12 @@ cudaError_t launch_step(const KParams<T>& p, const StepMaps& m, cudaStream_t s, 
 // columns instead of one and a little (96 x 170 x 170: depth 9, 1216 blocks, a step 55.6 us; depth 8, 68 before), and
 // short columns where a grid has few of them (48^3: depth 1 7.3 us, 2 8.2, 4 11.2).  Past three rounds only L/C + t a
 // plane matters, which the depth does not change, and it stays at kLongColumn.
-// Beside an interior kernel (FP32) the estimate is kept unless it takes shorter columns than kLongColumn for more than
-// two rounds: it counts every column at full depth, while most are the few planes of a z slab, which no depth changes
-// (a step of 328 x 376 x 306, 4-cell CPML, with depth 5, 2.3 rounds, 524 us, with 8 502; 260 x 252 x 240 with 6, 2.7 rounds, 224 and
-// 219; 280^3 and 296^3, 4-cell CPML, with 6 and 5, 1.9 and 1.8 rounds, 268 and 313, with 8 272 and 316).
+// Beside an interior kernel (FP32) the estimate is kept unless it takes shorter columns than kLongColumn where those would
+// fit in about one round, or in more than two rounds of its own: it counts every column at full depth, while most are the
+// few planes of a z slab, which no depth changes.  A step with the estimate's depth / with 8: 328 x 376 x 306, 4-cell CPML
+// (2.3 rounds of 5) 524 / 502 us; 260 x 252 x 240, 10 cells (2.7 rounds of 6) 224 / 219; 220 x 260 x 240, 2 cells (1.2 rounds
+// of 8) 195 / 186; 244 x 247 x 247, 4 cells (1.1) 200 / 192; 216^3 (0.9) 129.6 / 126.4; but 244^3 (1.3) 191 / 195, 252^3 (1.4)
+// 215 / 216, 296^3 (1.3) 313 / 316, 280^3 (1.5) 268 / 272, all with 4 cells.
 // Blocks of 128 threads, not 256: they spread more evenly over the SMs (FP64 32^3 step 12.2 -> 10.8 us,
 // 88^3 19.8 -> 15.5, 121 x 81 x 95 23.9 -> 23.2, 75 x 61 x 83 11.9 -> 11.5, 128^3 and up within 1%).
 void shell_shape(ShellBoxes& s, int type_bytes, size_t ncell, bool beside)
@@ -302,7 +304,8 @@ void shell_shape(ShellBoxes& s, int type_bytes, size_t ncell, bool beside)
             s.kz = kz;
         }
     }
-    if (beside && !f64 && s.kz < kLongColumn && blocks(s.kz) > 2 * C * sms) s.kz = kLongColumn;
+    if (beside && !f64 && s.kz < kLongColumn && (blocks(kLongColumn) <= C * sms * 6 / 5 || blocks(s.kz) > 2 * C * sms))
+        s.kz = kLongColumn;
     blocks(s.kz);
 }
 
