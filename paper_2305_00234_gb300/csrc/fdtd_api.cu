@@ -48,6 +48,7 @@ const double kPi = 3.14159265358979323846;
 constexpr int kGraphSteps = fdtd::kMaxSnap;   // one DFT block per captured graph
 constexpr int kChunkSteps = 512;
 constexpr size_t kInteriorCells32 = 9000000, kInteriorCells64 = 600000;   // see Solver::interior
+constexpr size_t kInteriorBox32One = 3000000;
 constexpr int kProfEvery = 4;                  // profiling times one DFT block in four
 
 struct Err {
@@ -432,14 +433,22 @@ struct Solver : SolverBase {
     // Whether the interior box is the fused kernel's, or the shell kernels take the whole grid, as they do on
     // grids below kInteriorCells32 / 64 cells: the fused kernel moves a third fewer bytes, but a block of it
     // is a chain of TMA latency, plane by plane, that a small launch cannot hide, while much of such a grid
-    // stays in L2.  Measured, one step with / without the fused kernel (FP32, three poles, 8-cell CPML): 64^3
-    // 18 / 12 us, 128^3 50 / 42, 160^3 85 / 76, 192^3 127 / 125, 128 x 256 x 256 158 / 151, 208^3 157 / 159, 224^3
-    // 193 / 195, 256^3 267 / 283.  FP64: 64^3 79 / 65, 80^3 106 / 104, 96^3 169 / 176.
+    // stays in L2.  Measured, one step with / without the fused kernel, three poles.  FP32, 8-cell CPML: 64^3 16.7 / 8.2
+    // us, 128^3 42.3 / 30.2, 160^3 72.8 / 64.8, 192^3 112.3 / 108.3, 208^3 135.2 / 133.7, 216^3 147.4 / 149.8, 224^3 168.6 /
+    // 167.9, 256^3 236.5 / 246.9.  FP64: 64^3 76 / 63, 80^3 99 / 102, 88^3 122.5 / 119.7, 96^3 157 / 161.
+    // Where the shell kernels are the one-cell ones (FP32, odd x CPML), which are slower, an interior box of kInteriorBox32One
+    // cells is enough (box of M cells, with / without): 144^3, 5-cell CPML (2.2) 64.8 / 60.9, 160^3 (2.6) 86.8 / 85.5, 168^3
+    // (3.8) 93.8 / 95.7, 176^3 (4.2) 101 / 108, 208^3 135 / 157; 9 cells: 160^3 (1.9) 91 / 87, 168^3 (2.75) 99.7 / 99.8,
+    // 192^3 (3.8) 126 / 133; 300 x 200 x 70, 5 cells (3.2) 79 / 82; the other way 96 x 300 x 240, 5 cells (3.8) 156 / 151.
     // An armed wait-timeout hook asks for the fused kernel's wait.
     bool interior() const
     {
         if (!fused || layout == 1) return false;
-        return layout == 2 || base.stall_ns > 0 || c->ncell >= (sizeof(T) == 4 ? kInteriorCells32 : kInteriorCells64);
+        if (layout == 2 || base.stall_ns > 0) return true;
+        if (sizeof(T) == 8) return c->ncell >= kInteriorCells64;
+        const int* b = base.ib;
+        return shell_all.pair ? c->ncell >= kInteriorCells32
+                              : (size_t)(b[1] - b[0]) * (b[3] - b[2]) * (b[5] - b[4]) >= kInteriorBox32One;
     }
     const fdtd::ShellBoxes& shell() const { return interior() ? shell_around : shell_all; }
 
