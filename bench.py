@@ -255,7 +255,7 @@ def kernel_hash():
     """Hash of the device-kernel sources with comments and whitespace removed (a comment edit does not
     change the kernels the DRAM counters were taken on)."""
     h = hashlib.sha256()
-    for f in ("fdtd_kernels.cuh", "fdtd_step.cuh", "fdtd_shell2.cuh", "fdtd_design2.cuh", "fdtd_dft.cuh", "fdtd_params.h"):
+    for f in ("fdtd_kernels.cuh", "fdtd_step.cuh", "fdtd_shell2.cuh", "fdtd_design2.cuh", "fdtd_dft.cuh", "fdtd_params.h", "fdtd_wait.h"):
         with open(os.path.join(ROOT, "paper_2305_00234_gb300", "csrc", f), "rb") as fh:
             t = fh.read().decode()
         t = re.sub(r"/\*.*?\*/", "", t, flags=re.S)

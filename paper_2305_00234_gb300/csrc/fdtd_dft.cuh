@@ -79,9 +79,8 @@ __global__ void __launch_bounds__(kDftThreads, sizeof(T) == 4 ? 5 : 2) dft_kerne
         o[2] = o[3] = -ph.y;                       // e (-sin) = -(e sin) exactly
     }
     __syncthreads();
-    if (!mbar_wait(bar, 0)) {
+    if (!patient_wait([&] { return mbar_try_wait(bar, 0); }, [] { return global_ns(); }, kWaitNs)) {
         if (tid == 0) atomicOr(d.ctl + 2, 4);
-        mbar_wait(bar, 0);                         // the block's copies, once more, before its memory goes
         return;
     }
     const bool on0 = tid < len, on1 = tid + kDftThreads < len;

@@ -26,6 +26,7 @@
 #include <climits>
 
 #include "fdtd_kernels.cuh"
+#include "fdtd_wait.h"
 
 namespace fdtd {
 
@@ -143,13 +144,7 @@ constexpr unsigned long long kWaitNs = 50ull * 1000 * 1000;   // a TMA plane arr
 // Wait for the phase of the given parity; false after limit_ns (or 2^26 tries) without completion.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, unsigned long long limit_ns = kWaitNs)
 {
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    for (int t = 0; t < (1 << 26); ++t) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (global_ns() - t0 > limit_ns) return false;
-    }
-    return false;
+    return bounded_wait([&] { return mbar_try_wait(bar, parity); }, [] { return global_ns(); }, limit_ns);
 }
 
 // ---- per-cell update rules ---------------------------------------------------------------------
