@@ -1192,6 +1192,7 @@ struct Solver : SolverBase {
         const int M = d.n_steps;
         const size_t ns = 3 * c->ngap;
         CK(fdtd::launch_paper_drive<T>(pm_gh, pm_drive, M, (int)ns, kEps0, c->work));
+        c->tim.launches++;
         // adjoint state to zero
         for (int f = 0; f < 4; ++f) CK(cudaMemsetAsync(pm_b.fld[f], 0, 3 * cs * sizeof(T), c->work));
         for (int cc = 0; cc < 3; ++cc)
@@ -1251,6 +1252,7 @@ struct Solver : SolverBase {
         const double dV = d.dx * d.dx * d.dx;
         void* dst = on_device ? out : (dtype == 1 ? (void*)grad : staging);
         CK(fdtd::launch_paper_scale(pm_gsum, dV, (long long)c->nd, dst, dtype, c->work));
+        c->tim.launches++;
         if (!on_device)
             CK(cudaMemcpyAsync(out, dst, c->nd * (dtype == 1 ? sizeof(double) : sizeof(float)), cudaMemcpyDeviceToHost, c->work));
         CK(cudaStreamSynchronize(c->work));
@@ -1384,7 +1386,7 @@ struct Solver : SolverBase {
             });
         }
         cudaGraphNode_t begin = nullptr, dftn = nullptr;
-        if (e == cudaSuccess) e = fdtd::graph_block_begin(g, &begin, p.ctl);
+        if (e == cudaSuccess && dp) e = fdtd::graph_block_begin(g, &begin, p.ctl);
         if (e == cudaSuccess)
             phase([&] {
                 cudaGraphNode_t n = nullptr;
@@ -1393,12 +1395,13 @@ struct Solver : SolverBase {
             });
         // the copy for the DFT comes before both the DFT and the step advance
         for (cudaGraphNode_t to : cur)
-            if (e == cudaSuccess) e = cudaGraphAddDependencies(g, &begin, &to, nullptr, 1);
+            if (e == cudaSuccess && begin) e = cudaGraphAddDependencies(g, &begin, &to, nullptr, 1);
         cudaGraphExec_t ex = nullptr;
         if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
         cudaGraphDestroy(g);
         if (e != cudaSuccess) {
             cudaGetLastError();
+            one_e = false;
             return nullptr;
         }
         return ex;
