@@ -37,14 +37,6 @@ __device__ __forceinline__ int slab_index(int l, int lo, int hi, int n)
     return l < lo ? l : (l >= n - hi ? lo + (l - (n - hi)) : -1);
 }
 
-template <typename T>
-__device__ __forceinline__ long long psi_index(const KParams<T>& p, int i, int j, int k, int a, int s)
-{
-    if (a == 0) return ((long long)k * p.ny + j) * p.W[0] + s;
-    if (a == 1) return ((long long)k * p.W[1] + s) * p.nx + i;
-    return ((long long)s * p.ny + j) * p.nx + i;
-}
-
 // CFS-CPML: psi <- b psi + c d ; derivative -> d / kappa + psi.
 #ifndef FDTD_PML4
 #define FDTD_PML4 1
@@ -67,19 +59,6 @@ __device__ __forceinline__ void pml_coef(const T* __restrict__ tab, int s, T& ki
     b = __ldg(tab + 4 * s + 1);
     c = __ldg(tab + 4 * s + 2);
 }
-
-template <typename T>
-__device__ __forceinline__ T stretch(T d, const T* __restrict__ tab, int s, T* psi)
-{
-    T kinv, b, c;
-    pml_coef(tab, s, kinv, b, c);
-    const T v = b * (*psi) + c * d;
-    *psi = v;
-    return d * kinv + v;
-}
-
-template <typename T>
-__device__ __forceinline__ T ldg_t(const T* p) { return __ldg(p); }
 
 #ifndef FDTD_ED_FASTDIV
 #define FDTD_ED_FASTDIV 1
@@ -114,15 +93,6 @@ __device__ __forceinline__ cpx<T> ldf(const cpx<T>* p)
     using V = typename vec2_of<T>::type;
     const V v = ldf<CG>(reinterpret_cast<const V*>(p));
     return cpx<T>{v.x, v.y};
-}
-
-template <typename T>
-__device__ __forceinline__ cpx<T> ldg_c(const cpx<T>* p)
-{
-    cpx<T> v;
-    v.re = __ldg(&p->re);
-    v.im = __ldg(&p->im);
-    return v;
 }
 
 // E update of one design sample of component C (blended), with Q^n:

@@ -27,14 +27,10 @@ static_assert(kShellKZ % kShell2PZ == 0, "column depth a multiple of the batch")
 
 __device__ __forceinline__ float2 p_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
 
-// L2 prefetch of the field rows a column needs FDTD_SHELL2_PF_H / _E planes ahead in the H / E kernel (0:
-// none): the loads of the coming planes then find their lines in L2 instead of waiting on HBM, without
-// holding registers.
-#ifndef FDTD_SHELL2_PF_H
-#define FDTD_SHELL2_PF_H 0
-#endif
+// L2 prefetch of the field rows a column needs FDTD_SHELL2_PF_E planes ahead in the E kernel (0: none): the loads of the
+// coming planes then find their lines in L2 instead of waiting on HBM, without holding registers.
 #ifndef FDTD_SHELL2_PF_E
-#define FDTD_SHELL2_PF_E 1   // measured: E kernel 0.0616 -> 0.0610 ms on the config-2 grid; the H kernel slows
+#define FDTD_SHELL2_PF_E 1   // measured: E kernel 0.0616 -> 0.0610 ms on a 256^3 grid; in the H kernel it slows
 #endif
 __device__ __forceinline__ void pf_l2(const float* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
@@ -166,17 +162,6 @@ __global__ void __launch_bounds__(kShellNT, FDTD_SHELL2_MINB) shell_h2_kernel(co
             if (k >= cl.k1) continue;
             const unsigned id = (unsigned)k * plane + col;
             const bool zp = k + 1 < p.nz;
-            if (FDTD_SHELL2_PF_H > 0 && k + FDTD_SHELL2_PF_H < cl.k1) {
-                const unsigned ip = id + FDTD_SHELL2_PF_H * plane;
-                pf_l2(p.H[0] + ip);
-                pf_l2(p.H[1] + ip);
-                pf_l2(p.H[2] + ip);
-                if (k + FDTD_SHELL2_PF_H + 1 < p.nz) {
-                    pf_l2(E0 + ip + plane);
-                    pf_l2(E1 + ip + plane);
-                    pf_l2(E2 + ip + plane);
-                }
-            }
             ex0[r] = r == 0 ? exc : exz[r - 1];
             ey0[r] = r == 0 ? eyc : eyz[r - 1];
             ez0[r] = ldp(E2 + id);

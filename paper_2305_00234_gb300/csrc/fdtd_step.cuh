@@ -165,10 +165,9 @@ __device__ __forceinline__ void h_cheap(const HIn<T>& a, T cneg, bool tf, T einc
     hz = fma_rn(cneg, sub_rn(sub_rn(a.eyx, a.ey0), sub_rn(a.exy, a.ex0)), a.hoz);
 }
 
-// E^{n+1} of one cell from the six H differences (unscaled) and E^n.  Cells outside the slabs, off
-// the walls and outside the source box take E = ca E + (cb/dx)((a - b) - (c - d)); the others scale
-// each difference by 1/dx, stretch the slab terms (psi_E in place), add the point-source drive and
-// keep the wall-tangential components at zero.
+// E^{n+1} of one interior cell (outside the slabs, off the walls) from the six H differences (unscaled) and E^n:
+// E = ca E + (cb/dx)((a - b) - (c - d)); inside the source box each difference is scaled by 1/dx and the point-source
+// drive added.
 template <typename T>
 struct EOut {
     T ex, ey, ez;
@@ -179,48 +178,22 @@ __device__ __forceinline__ EOut<T> e_cell(const KParams<T>& p, int i, int j, int
                                           T rxa, T rxb, T rya, T ryb, T rza, T rzb)
 {
     const bool tf = i == p.tfsf_i0;                                        // H_y(i0-1/2) is scattered field
-    const int sx = slab_index(i, p.cpl[0], p.cph[0], p.nx);
-    const int sy = slab_index(j, p.cpl[1], p.cph[1], p.ny);
-    const int sz = slab_index(k, p.cpl[2], p.cph[2], p.nz);
-    const bool src = p.nb > 0 && in_box(p.sb, i, j, k);
     EOut<T> e;
-    if (sx < 0 && sy < 0 && sz < 0 && !src && i > 0 && j > 0 && k > 0) {
+    if (!(p.nb > 0 && in_box(p.sb, i, j, k))) {
         e.ex = p.bg_ca[0] * ex0 + p.bg_cbi[0] * (rxa - rxb);
         e.ey = p.bg_ca[1] * ey0 + p.bg_cbi[1] * (rya - ryb);
         e.ez = p.bg_ca[2] * ez0 + p.bg_cbi[2] * ((tf ? rza - hinc_n : rza) - rzb);
         return e;
     }
     const T idx = p.inv_dx;
-    T xa = rxa * idx, xb = rxb * idx, ya = rya * idx, yb = ryb * idx, za = rza * idx, zb = rzb * idx;
+    T za = mul_rn(rza, idx);
     if (tf) za -= hinc_n * idx;
-    if (sy >= 0) {
-        const long long q = psi_index(p, i, j, k, 1, sy);
-        xa = stretch(xa, p.pmlE[1], sy, p.psiE[0][0] + q);
-        zb = stretch(zb, p.pmlE[1], sy, p.psiE[2][1] + q);
-    }
-    if (sz >= 0) {
-        const long long q = psi_index(p, i, j, k, 2, sz);
-        xb = stretch(xb, p.pmlE[2], sz, p.psiE[0][1] + q);
-        ya = stretch(ya, p.pmlE[2], sz, p.psiE[1][0] + q);
-    }
-    if (sx >= 0) {
-        const long long q = psi_index(p, i, j, k, 0, sx);
-        yb = stretch(yb, p.pmlE[0], sx, p.psiE[1][1] + q);
-        za = stretch(za, p.pmlE[0], sx, p.psiE[2][0] + q);
-    }
-    T dxv = xa - xb, dyv = ya - yb, dzv = za - zb;
-    if (src) {
-        dxv += point_drive(p, i, j, k, 0, n);
-        dyv += point_drive(p, i, j, k, 1, n);
-        dzv += point_drive(p, i, j, k, 2, n);
-    }
+    const T dxv = sub_rn(mul_rn(rxa, idx), mul_rn(rxb, idx)) + point_drive(p, i, j, k, 0, n);
+    const T dyv = sub_rn(mul_rn(rya, idx), mul_rn(ryb, idx)) + point_drive(p, i, j, k, 1, n);
+    const T dzv = sub_rn(za, mul_rn(rzb, idx)) + point_drive(p, i, j, k, 2, n);
     e.ex = p.bg_ca[0] * ex0 + p.bg_cb[0] * dxv;
     e.ey = p.bg_ca[1] * ey0 + p.bg_cb[1] * dyv;
     e.ez = p.bg_ca[2] * ez0 + p.bg_cb[2] * dzv;
-    const bool im = i > 0, jm = j > 0, km = k > 0;
-    if (!(jm && km)) e.ex = ex0;   // PEC walls: components tangential to a wall at index 0 stay zero
-    if (!(km && im)) e.ey = ey0;
-    if (!(im && jm)) e.ez = ez0;
     return e;
 }
 
