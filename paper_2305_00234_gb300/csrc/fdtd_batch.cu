@@ -68,8 +68,8 @@ __device__ __forceinline__ bool wait_count(const unsigned* p, unsigned need, con
     return false;
 }
 
-// DFT fold of one voxel over steps n0 .. n0 + cnt - 1 (the arithmetic of dft_voxel, the same sums in
-// the same order) one component and frequency at a time, which keeps few values live: snapshots are
+// DFT fold of one voxel over steps n0 .. n0 + cnt - 1 (dft_kernel's sums in the same
+// order), one component and frequency at a time, which keeps few values live: snapshots are
 // re-read from L2 per frequency instead of being held in registers.
 template <typename T>
 __device__ __forceinline__ void dft_voxel_lean(const DParams<T>& d, long long v, int n0, int cnt)

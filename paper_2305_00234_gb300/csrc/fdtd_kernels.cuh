@@ -11,8 +11,8 @@
 // kernel evaluates the structure of Eq. (Gradient_analytic) per voxel (or per E sample with the
 // per-sample density layout) with a deterministic warp-shuffle reduction of its squared norm.
 //
-// Thread layout of the per-cell kernels: blocks of (32, 8) threads over (x, y); x is the fastest
-// array axis, so each warp reads and writes 128 contiguous bytes per field (FP32).
+// Thread layout of the per-cell kernels: a block takes 256 (design) or 128 (shell) consecutive (x, y) columns or
+// column pairs; x is the fastest array axis, so each warp reads and writes 128 or 256 contiguous bytes per field (FP32).
 //
 // The step index lives in device memory so that a CUDA graph of K steps can be replayed: ctl[0] is the
 // first step of the graph and every launch's step is ctl[0] + n_off (a launch parameter).  Next to the first
@@ -225,8 +225,8 @@ __device__ __forceinline__ cpx<T> ld_pre(const cpx<T>* p)
 // ---------------------------------------------------------------------------------------------
 // E update inside the working box.  A thread owns one component c of the (x, y) column of a block
 // of p.edz planes (blockIdx.z = 3 zc + c, so the three components of a plane run in neighbouring
-// blocks and share its H in L2; the per-block set-up and step-advance bookkeeping are paid once per
-// p.edz planes) and handles its planes kEdPZ at a time, every load of a batch (the pole currents
+// blocks and share its H in L2; the per-column set-up is paid once per p.edz
+// planes) and handles its planes kEdPZ at a time, every load of a batch (the pole currents
 // included) before any store: blended CCPR update of the design samples, background
 // update of the gap samples and of samples outside their component's sample box, point sources,
 // the E snapshot for the blocked DFT and the paper-mode records.  The working box lies outside the

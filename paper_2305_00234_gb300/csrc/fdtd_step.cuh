@@ -556,9 +556,9 @@ __device__ __forceinline__ T stretch_v(T d, const T* __restrict__ tab, int s, T&
 }
 
 // H^{n+1/2} of one column (x, y), planes [k0, k1) (at most kShellKZ of them): every cell update of
-// the shell, CPML psi_H included.  Within a batch every load is issued before any store (the buffers
-// it writes are not the ones it reads); E_x, E_y of the plane above a batch carry over as the next
-// batch's own.  CG: state loads bypass L1 (for a persistent kernel whose earlier work items on the
+// the shell, CPML psi_H included.  Within a batch every load is issued before any store.  The buffers it writes are
+// other ones than it reads or, in place, the same: H and psi_H are read only at the cells the thread itself writes, each
+// before its store.  E_x, E_y of the plane above a batch carry over as the next batch's own.  CG: state loads bypass L1 (for a persistent kernel whose earlier work items on the
 // same SM may hold stale lines).  PDL: the caller has not waited for the phase before; the first batch's
 // H and psi_H loads come first.
 template <typename T, bool CG, bool PDL = false, int P = kShellPZ<T>>
@@ -686,7 +686,7 @@ __global__ void __launch_bounds__(kShellNT, sizeof(T) == 8 ? 4 : FDTD_SHELL_MINB
 
 // E^{n+1} of the cells of one column (x, y), planes [k0, k1), that lie outside the working box, from
 // H^{n+1/2} of the whole grid (after every H update of the step); loads first within a batch, like
-// h_column, with H_x, H_y of the plane below a batch carried over.  Returns the largest |E| sum seen
+// h_column, and E and psi_E read only at the thread's own cells; H_x, H_y of the plane below a batch are carried over.  Returns the largest |E| sum seen
 // on a checked step (0 otherwise).  PDL: the caller has not waited for the phase before; the first batch's
 // E and psi_E loads come first.
 template <typename T, bool CG, bool PDL = false, int P = kShellPZ<T>>
