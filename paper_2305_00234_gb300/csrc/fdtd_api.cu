@@ -433,13 +433,14 @@ struct Solver : SolverBase {
     // Whether the interior box is the fused kernel's, or the shell kernels take the whole grid, as they do on
     // grids below kInteriorCells32 / 64 cells: the fused kernel moves a third fewer bytes, but a block of it
     // is a chain of TMA latency, plane by plane, that a small launch cannot hide, while much of such a grid
-    // stays in L2.  Measured, one step with / without the fused kernel, three poles.  FP32, 8-cell CPML: 64^3 16.7 / 8.2
-    // us, 128^3 42.3 / 30.2, 160^3 72.8 / 64.8, 192^3 112.3 / 108.3, 208^3 135.2 / 133.7, 216^3 147.4 / 149.8, 224^3 168.6 /
-    // 167.9, 256^3 236.5 / 246.9.  FP64: 64^3 76 / 63, 80^3 99 / 102, 88^3 122.5 / 119.7, 96^3 157 / 161.
+    // stays in L2.  Measured, one step with / without the fused kernel, three poles, design boxes of about half the extents.
+    // FP32, 8-cell CPML: 64^3 16.0 / 7.9 us, 128^3 42.5 / 30.3, 160^3 73.3 / 64.9, 192^3 112.5 / 108.2, 208^3 135.1 / 134.4,
+    // 216^3 147.6 / 150.0, 224^3 169.4 / 168.0, 256^3 236.4 / 247.4.  FP64: 64^3 76 / 63, 80^3 99 / 102, 88^3 122.5 / 119.8, 96^3
+    // 157.6 / 161.2.
     // Where the shell kernels are the one-cell ones (FP32, odd x CPML), which are slower, an interior box of kInteriorBox32One
-    // cells is enough (box of M cells, with / without): 144^3, 5-cell CPML (2.2) 64.8 / 60.9, 160^3 (2.6) 86.8 / 85.5, 168^3
-    // (3.8) 93.8 / 95.7, 176^3 (4.2) 101 / 108, 208^3 135 / 157; 9 cells: 160^3 (1.9) 91 / 87, 168^3 (2.75) 99.7 / 99.8,
-    // 192^3 (3.8) 126 / 133; 300 x 200 x 70, 5 cells (3.2) 79 / 82; the other way 96 x 300 x 240, 5 cells (3.8) 156 / 151.
+    // cells is enough (box of M cells, with / without): 144^3, 5-cell CPML (2.2) 64.3 / 61.0, 160^3 (2.6) 86.8 / 85.3, 168^3
+    // (3.8) 93.8 / 95.7, 176^3 (4.2) 101.6 / 108.8, 208^3 152 / 174; 9 cells: 160^3 (1.9) 91.3 / 87.2, 168^3 (2.75) 99.7 / 100.0,
+    // 192^3 (3.8) 139 / 147; 300 x 200 x 70, 5 cells (3.2) 80 / 82; the other way 96 x 300 x 240, 5 cells (3.8) 156 / 151.
     // An armed wait-timeout hook asks for the fused kernel's wait.
     bool interior() const
     {

@@ -267,12 +267,12 @@ cudaError_t launch_step(const KParams<T>& p, const StepMaps& m, cudaStream_t s, 
 // columns instead of one and a little (96 x 170 x 170: depth 9, 1216 blocks, a step 55.6 us; depth 8, 68 before), and
 // short columns where a grid has few of them (48^3: depth 1 7.3 us, 2 8.2, 4 11.2).  Past three rounds only L/C + t a
 // plane matters, which the depth does not change, and it stays at kLongColumn.
-// Beside an interior kernel (FP32) the estimate is kept unless it takes shorter columns than kLongColumn and those would
-// not leave a second round nearly empty (1.2 to 1.6 rounds of blocks): it counts every column at full depth, while most are
+// Beside an interior kernel (FP32) the estimate is kept unless it takes shorter columns than kLongColumn in more than one
+// round and those of kLongColumn would not leave a round nearly empty (1.2 to 1.6 rounds of blocks): it counts every column at full depth, while most are
 // the few planes of a z slab, which no depth changes.  A step with the estimate's depth / with 8 (rounds of 8): 216^3, 4-cell
 // CPML (0.9) 129.6 / 126.4 us; 244 x 247 x 247, 4 (1.1) 200 / 192; 220 x 260 x 240, 2 (1.2) 195 / 186; 328 x 376 x 306, 4 (1.8)
 // 524 / 502; 260 x 252 x 240, 10 (2.3) 224 / 219; but 296^3, 4 (1.3) 313 / 316, 244^3, 4 (1.3) 191 / 195, 252^3, 4 (1.4) 215 / 216,
-// 228 x 204 x 224, 8 (1.5) 195.4 / 196.5, 280^3, 4 (1.5) 268 / 272.
+// 228 x 204 x 224, 8 (1.5) 195.4 / 196.5, 280^3, 4 (1.5) 268 / 272, and 128^3, 8 (0.9 rounds of the estimate's 4) 42.3 / 47.4.
 // Blocks of 128 threads, not 256: they spread more evenly over the SMs (FP64 32^3 step 12.2 -> 10.8 us,
 // 88^3 19.8 -> 15.5, 121 x 81 x 95 23.9 -> 23.2, 75 x 61 x 83 11.9 -> 11.5, 128^3 and up within 1%).
 void shell_shape(ShellBoxes& s, int type_bytes, size_t ncell, bool beside)
@@ -304,8 +304,8 @@ void shell_shape(ShellBoxes& s, int type_bytes, size_t ncell, bool beside)
             s.kz = kz;
         }
     }
-    if (beside && !f64 && s.kz < kLongColumn) {
-        const unsigned n = blocks(kLongColumn), round = C * sms;
+    if (const unsigned round = C * sms; beside && !f64 && s.kz < kLongColumn && blocks(s.kz) > round) {
+        const unsigned n = blocks(kLongColumn);
         if (n <= round * 6 / 5 || n >= round * 8 / 5) s.kz = kLongColumn;
     }
     blocks(s.kz);

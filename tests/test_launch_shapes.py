@@ -35,10 +35,11 @@ def around(n, ib):
             (0, n[0], ib[3], n[1], ib[4], ib[5]), (0, ib[0], ib[2], ib[3], ib[4], ib[5]), (ib[1], n[0], ib[2], ib[3], ib[4], ib[5])]
 
 
-# beside an interior kernel: columns shorter than 8 planes only where 8 would make 1.2 to 1.6 rounds of blocks
+# beside an interior kernel: columns shorter than 8 planes only in one round, or where 8 would make 1.2 to 1.6 rounds of blocks
 @pytest.mark.parametrize("n,ib,kz", [((328, 376, 306), (8, 324, 5, 372, 5, 302), 8), ((260, 252, 240), (16, 240, 11, 235, 11, 230), 8),
                                      ((280, 280, 280), (8, 264, 5, 276, 5, 276), 6), ((244, 247, 247), (8, 232, 5, 243, 5, 243), 8),
                                      ((244, 244, 244), (8, 232, 5, 229, 5, 240), 5), ((228, 204, 224), (16, 208, 9, 185, 9, 216), 4),
+                                     ((128, 128, 128), (32, 120, 9, 120, 9, 120), 4),
                                      ((220, 260, 240), (8, 200, 3, 258, 3, 238), 8), ((296, 296, 296), (16, 272, 9, 281, 9, 288), 9)])
 def test_columns_beside_an_interior_kernel(n, ib, kz):
     assert shape(around(n, ib), True, 4, n[0] * n[1] * n[2], True)[0] == kz
