@@ -804,7 +804,9 @@ struct Solver : SolverBase {
     // or whole lines, in every tile row's stores: with x0 at 48 or 80 bytes from a line the kernel wrote half
     // sectors that two tiles share, and ran at 4.7 TB/s instead of 6.2 on a 512 x 512 x 384 grid, a step of
     // which went from 1909 to 1658 us; 256^3 with a 12-cell CPML, x0 at 64 and at 128 bytes: 275 and 271 us;
-    // 208^3, whose rows are no multiple of 128 bytes, x0 at 64 and at 128 bytes: 157 and 165 us), planes cpml_z_low + 1
+    // 208^3, whose rows are no multiple of 128 bytes, x0 at 64 and at 128 bytes: 157 and 165 us).  Where the x rows are no
+    // multiple of 32 bytes, half of them start within a sector anyway, and x0 is a multiple of 16 if that gives a wider box (204 x 240
+    // x 230, 8-cell CPML, x0 at 48 and at 64 bytes: 161 and 181 us; 252 x 240 x 230, 16 cells: 202 and 218).  Planes cpml_z_low + 1
     // .. nz - cpml_z_high - 1 (the plane below the first one is outside the slab too), at least one whole
     // tile each way.  Toward the +x and +y slabs the box ends in a partial tile column or row (an even
     // number of x cells; the kernel leaves the cells beyond to the shell) when that tile holds at least
@@ -826,20 +828,24 @@ struct Solver : SolverBase {
     void split_grid(KParams<T>& p)
     {
         const fdtd_grid_desc& d = c->d;
-        int X0 = 0;
-        for (int line : {128, 32, 16}) {   // the largest alignment that leaves room for a tile
-            const int xa = line / (int)sizeof(T);
-            if (line == 128 && d.nx % xa) continue;
-            X0 = std::max((std::max(p.cpl[0] + 1, 1) + xa - 1) / xa * xa, 4);
-            if (d.nx - p.cph[0] - X0 >= fdtd::kTX) break;
+        auto x_start = [&](int xa) { return std::max((std::max(p.cpl[0] + 1, 1) + xa - 1) / xa * xa, 4); };
+        auto tiled = [](int w) {   // cells of a width that whole and mostly full tiles take
+            const int r = (w & ~1) % fdtd::kTX;
+            return w / fdtd::kTX * fdtd::kTX + (FDTD_PARTIAL_TILES && r >= FDTD_PARTIAL_MIN_X ? r : 0);
+        };
+        int X0 = x_start(16 / (int)sizeof(T));
+        const int w16 = d.nx - p.cph[0] - X0;
+        for (int line : {32, 128}) {   // the largest alignment that leaves room for a tile
+            const int xa = line / (int)sizeof(T), w = d.nx - p.cph[0] - x_start(xa);
+            if (w >= fdtd::kTX && (d.nx % xa == 0 || (line == 32 && tiled(w) >= tiled(w16)))) X0 = x_start(xa);
         }
         const int Y0 = std::max(p.cpl[1] + 1, 1), Z0 = p.cpl[2] + 1;
         const int wx = d.nx - p.cph[0] - X0, wy = d.ny - p.cph[1] - Y0;   // widths up to the +x / +y slabs
         const int Z1 = d.nz - p.cph[2];
         fused = ((size_t)d.nx * sizeof(T)) % 16 == 0 && wx >= fdtd::kTX && wy >= fdtd::kTY && Z1 > Z0 &&
                 tensor_map_encoder() != nullptr;
-        const int rx = (wx & ~1) % fdtd::kTX, ry = wy % fdtd::kTY;   // cells of a partial last tile
-        const int X1 = X0 + wx / fdtd::kTX * fdtd::kTX + (FDTD_PARTIAL_TILES && rx >= FDTD_PARTIAL_MIN_X ? rx : 0);
+        const int ry = wy % fdtd::kTY;   // rows of a partial last tile
+        const int X1 = X0 + tiled(wx);
         const int Y1 = Y0 + wy / fdtd::kTY * fdtd::kTY + (FDTD_PARTIAL_TILES && ry >= FDTD_PARTIAL_MIN_Y ? ry : 0);
         const int ntx = (X1 - X0 + fdtd::kTX - 1) / fdtd::kTX, nty = (Y1 - Y0 + fdtd::kTY - 1) / fdtd::kTY;
         const int ib[6] = {X0, X1, Y0, Y1, Z0, Z1};

@@ -5,8 +5,10 @@ method's; between checkpoint intervals those of test_paper_graphs_gpu."""
 import numpy as np
 import pytest
 
+import synth
 import test_parity_gpu as parity
 from parity_util import TOL, rel
+from synth import base_desc, vacuum
 from test_paper_mode_gpu import _case, _oracle
 from test_parity_gpu import compare, gpu, run_oracle  # noqa: F401
 
@@ -96,4 +98,18 @@ def test_layout_changes_between_paper_passes(gpu, first, second):  # noqa: F811
     assert abs(p.paper_forward(checkpoint_steps=33) - F) <= 1e-12 * abs(F)
     assert rel(p.paper_gradient(pole_pairing=1), g) <= 1e-12
     assert np.isfinite(p.forward()[0])                            # a plain run after them
+    p.close()
+
+
+# x rows of no multiple of 32 bytes: the box starts on 16 bytes where that keeps a mostly full last tile column
+@pytest.mark.parametrize("prec,nx,cpml_x,box_x", [(32, 76, 8, (12, 68)), (32, 68, 8, (16, 48)), (64, 90, 12, (14, 78)),
+                                                   (64, 78, 5, (8, 72))])
+def test_box_start_of_odd_rows(gpu, prec, nx, cpml_x, box_x):  # noqa: F811
+    d = base_desc(nx, 42, 37, n_steps=420, cpml=(cpml_x, cpml_x, 4, 7, 5, 3), precision=prec, design=(22, 18, 15), gap=(2, 2, 2),
+                  lambdas_nm=(500.0, 650.0), src_kind=1, src_pos=(cpml_x + 3, 0, 0))
+    w = dict(desc=d, bg=vacuum(), m1=vacuum(), m2=synth.drude_lorentz_metal(23, 3), gamma=1e6,
+             rho=synth.smooth_rho(synth.box_shape(d["design_box"]), 23, 2.0))
+    p = problem(gpu, w, 2)
+    assert p.timings()["interior_cells"] == (box_x[1] - box_x[0]) * 30 * 28
+    compare(run(p, w), run_oracle(w), prec)
     p.close()
